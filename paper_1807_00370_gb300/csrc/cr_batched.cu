@@ -122,6 +122,29 @@ __device__ inline void make_level_args(LevelArgs &a, const BatchArgs &ba, const 
     a.dbg = ba.dbg;
 }
 
+// One chunk in the form of its block size (the form the level kernels take).
+template <int MT>
+__device__ __forceinline__ void factor_of(const LevelArgs &a, int64_t c, unsigned char *smem) {
+    if constexpr (Forms<MT, double>::fma) {
+        if (!split_form(a.m, 8)) return factor_chunk<MT, double>(a, c, smem);
+    }
+    if constexpr (Forms<MT, double>::split) factor_chunk_split<MT>(a, c, smem);
+}
+template <int MT>
+__device__ __forceinline__ void solve_down_of(const LevelArgs &a, int64_t c, int cc, unsigned char *smem) {
+    if constexpr (Forms<MT, double>::fma) {
+        if (!split_form(a.m, 8)) return solve_down_chunk<MT, double>(a, c, cc, smem);
+    }
+    if constexpr (Forms<MT, double>::split) solve_down_chunk_split<MT>(a, c, cc, smem);
+}
+template <int MT>
+__device__ __forceinline__ void solve_up_of(const LevelArgs &a, int64_t c, int cc, unsigned char *smem) {
+    if constexpr (Forms<MT, double>::fma) {
+        if (!split_form(a.m, 8)) return solve_up_chunk<MT, double>(a, c, cc, smem);
+    }
+    if constexpr (Forms<MT, double>::split) solve_up_chunk_split<MT>(a, c, cc, smem);
+}
+
 // The whole classic cyclic reduction of one system, run by one CTA.  The
 // level arguments live in shared memory (sa) so that they do not hold
 // registers across the chunk loops.
@@ -140,7 +163,7 @@ __device__ __noinline__ void run_system(const BatchArgs &ba, const SysDesc &d, i
         }
         __syncthreads();
         for (int64_t c = 0, nc = crs_num_ctas(sa.no, sa.nb); c < nc; ++c) {
-            factor_chunk<MT, double>(sa, c, smem);
+            factor_of<MT>(sa, c, smem);
             __syncthreads();
         }
         if (threadIdx.x == 0) {
@@ -151,7 +174,7 @@ __device__ __noinline__ void run_system(const BatchArgs &ba, const SysDesc &d, i
         const int ncc = (k + sa.kc - 1) / sa.kc;
         for (int64_t c = 0, nc = crs_num_ctas(sa.no, sa.nb); c < nc; ++c)
             for (int cc = 0; cc < ncc; ++cc) {
-                solve_down_chunk<MT, double>(sa, c, cc, smem);
+                solve_down_of<MT>(sa, c, cc, smem);
                 __syncthreads();
             }
     }
@@ -166,7 +189,7 @@ __device__ __noinline__ void run_system(const BatchArgs &ba, const SysDesc &d, i
         const int ncc = (k + sa.kc - 1) / sa.kc;
         for (int64_t c = 0, nc = crs_num_ctas(sa.no, sa.nb); c < nc; ++c)
             for (int cc = 0; cc < ncc; ++cc) {
-                solve_up_chunk<MT, double>(sa, c, cc, smem);
+                solve_up_of<MT>(sa, c, cc, smem);
                 __syncthreads();
             }
     }

@@ -1297,3 +1297,27 @@ __device__ __forceinline__ void solve_up_chunk(const LevelArgsT<R> &a, int64_t c
 }
 
 }  // namespace crs
+
+#include "cr_core64.cuh"
+
+namespace crs {
+
+// The split forms as the kernels call them: blocks that fill their class need
+// no bounds in the tile loads.
+template <int MT>
+__device__ __forceinline__ void factor_chunk_split(const LevelArgs &a, int64_t chunk, unsigned char *smem) {
+    if (a.m == MT) factor_split<MT, true>(a, chunk, smem);
+    else factor_split<MT, false>(a, chunk, smem);
+}
+template <int MT>
+__device__ __forceinline__ void solve_down_chunk_split(const LevelArgs &a, int64_t chunk, int cchunk, unsigned char *smem) {
+    if (a.m == MT) solve_down_split<MT, true>(a, chunk, cchunk, smem);
+    else solve_down_split<MT, false>(a, chunk, cchunk, smem);
+}
+template <int MT>
+__device__ __forceinline__ void solve_up_chunk_split(const LevelArgs &a, int64_t chunk, int cchunk, unsigned char *smem) {
+    if (a.m == MT) solve_up_split<MT, true>(a, chunk, cchunk, smem);
+    else solve_up_split<MT, false>(a, chunk, cchunk, smem);
+}
+
+}  // namespace crs

@@ -1,0 +1,683 @@
+// cr_core64.cuh -- the FP64 level steps of the blocks of split_form,
+// run by one CTA on one chunk of a level, with every product on the tensor
+// cores (cr_split.cuh).
+//
+// The factor keeps X = L^{-1} of every odd block in place of L, so that all
+// triangular solves are products: Z = X [B_l | B_r^H], r = X y, x = X^H w.  With
+// FP64 FMAs the solves, Z^H Z and the sweeps' products were 95% of the FP64
+// instructions of a step, on a pipe of 2 FMA per clock per SM; here FP64
+// instructions are left in the Cholesky factorisation with its inverse and in
+// one rounding per result.
+//
+// An inverse of L is as good as substitution where it is multiplied exactly:
+// the rounding errors of X are those of the substitution on the unit vectors
+// (L X = I + E, |E| <= m u |L| |X|), and a product with X adds one rounding of
+// its result where a substitution adds one per term.
+//
+// Tiles are 8 x 8; blocks whose m is no multiple of 8 are padded with zeros in
+// registers.  Every result depends on the block's data alone, not on the chunk
+// size, the threads or the right-hand-side chunk, so the level kernels, the
+// batched kernel and the allocation-free path agree bit for bit.
+#pragma once
+#include "cr_split.cuh"
+
+namespace crs {
+
+// Which blocks take these forms: those that fill their tiles well enough.  A
+// block of m <= 4 would fill a quarter of a fragment; at m = 5 the padding to
+// 8 x 8 costs more than the FMAs (factor and solve at N = 100003, k = 3: 815 + 1076
+// against 595 + 800 us), and so does that of m = 9 .. 11 to 16 x 16 (factor at
+// m = 9, N = 65842: 2602 against 1761 us; at m = 12, N = 27776: 1432 against 1622).
+__host__ __device__ constexpr bool split_form(int m, size_t rsize) { return rsize == 8 && (m >= 12 || m == 7 || m == 8); }
+// The classes that have blocks of either kind.
+template <int MT, class R> struct Forms {
+    static constexpr bool split = sizeof(R) == 8 && MT >= 8;
+    static constexpr bool fma = sizeof(R) == 4 || MT <= 16;
+};
+
+// Shared memory of a chunk, in complex entries per odd block.  Odd strides
+// keep the accesses of consecutive blocks and rows in different banks.
+template <int MT> struct Split64 {
+    static constexpr int LDZ = 2 * MT + 1;          // row of Z
+    static constexpr int SL = Tri<MT>::n | 1;       // packed triangle
+    static constexpr int SC = 9;                    // one column of an 8 x 8 diagonal block
+    static constexpr int SU = MT > 8 ? 8 * MT : 0;  // one row of blocks of -X_II^{-1} X (see inverse_chunk)
+};
+__host__ __device__ constexpr size_t factor64_entries(int mt) {
+    return (size_t)(((mt * (mt + 1) / 2) | 1) + mt * (2 * mt + 1) + 9 + (mt > 8 ? 8 * mt : 0));
+}
+
+// Row of entry f of a packed 8 x 8 lower triangle.
+__device__ __forceinline__ int tri8_row(int f) {
+    constexpr unsigned kStarts = 1u << 1 | 1u << 3 | 1u << 6 | 1u << 10 | 1u << 15 | 1u << 21 | 1u << 28;
+    return f >= 28 ? 7 : __popc(kStarts & ((2u << f) - 1u));
+}
+
+// X = L^{-1} of the diagonal blocks o .. o + w - 1 (w <= 8) of A_b = L L^H (packed
+// lower in sL, in place) for the blocks b < nbh of a chunk, with the breakdown
+// test of every pivot.  Right-looking: with column c of L final, every later row
+// r takes l_r times (the conjugate of) column c of L off its trailing entries
+// and l_r times row c of X off its entries of X; column c of L is not needed
+// after that, so X takes its place (a Gauss-Jordan step).  A step is two
+// barriers: the scaling of column c and of row c of X; the updates, one entry
+// per thread, and meanwhile in a warp of its own (about as long as the other
+// warps' updates) the next pivot.  Consecutive threads take consecutive blocks.
+// Ends with __syncthreads().
+template <int MT>
+__device__ __forceinline__ void chol_inv8(const LevelArgs &a, int64_t t0, z2 *sL, z2 *sC, int nbh, int o, int w) {
+    constexpr int SL = Split64<MT>::SL, SC = Split64<MT>::SC;
+    const int NT = blockDim.x, tid = threadIdx.x;
+    const int npiv = NT >= 64 ? 32 : 0;       // threads kept for the pivots
+    auto at = [&](int r, int c) { return tri(o + r, o + c); };
+    auto pivot = [&](int b, int c, double d) {
+        if (!(d > 0.0)) report_fail(a.status, a.level, report_index(a, 2 * (t0 + b)));
+        sL[b * SL + at(c, c)] = zmk(rsq(d), 0.0);
+    };
+    const int pstep = npiv ? npiv : NT;
+    const bool piv = tid < pstep;
+    if (piv)
+        for (int b = tid; b < nbh; b += pstep) pivot(b, 0, sL[b * SL + at(0, 0)].x);
+    const int q1 = min(nbh, NT), b1 = tid % q1, f1 = tid / q1, s1 = NT / q1;
+    const int nu = NT - npiv, q2 = min(nbh, nu), ut = tid - npiv, b2 = ut % q2, f2 = ut / q2, s2 = nu / q2;
+    const int ntri = w * (w + 1) / 2;
+    for (int c = 0; c < w; ++c) {
+        __syncthreads();
+        if (f1 < s1 && f1 < w)
+            for (int b = b1; b < nbh; b += q1) {
+                z2 *Lb = sL + b * SL;
+                const double iv = Lb[at(c, c)].x;
+                for (int i = f1; i < w; i += s1) {
+                    if (i > c) sC[b * SC + i] = zscale(Lb[at(i, c)], iv);
+                    else if (i < c) Lb[at(c, i)] = zscale(Lb[at(c, i)], iv);
+                }
+            }
+        __syncthreads();
+        if (c + 1 == w) break;
+        if (piv)
+            for (int b = tid; b < nbh; b += pstep) {
+                const z2 l = sC[b * SC + c + 1];
+                double d = sL[b * SL + at(c + 1, c + 1)].x;
+                d = fma(-l.x, l.x, d);
+                d = fma(-l.y, l.y, d);
+                pivot(b, c + 1, d);
+            }
+        if (ut >= 0 && f2 < s2)
+            for (int b = b2; b < nbh; b += q2) {
+                z2 *Lb = sL + b * SL;
+                const z2 *Cb = sC + b * SC;
+                for (int f = tri(c + 1, 0) + f2; f < ntri; f += s2) {
+                    const int r = tri8_row(f), j = f - tri(r, 0);
+                    if (j == c + 1 && r == c + 1) continue;             // the next pivot
+                    const z2 l = Cb[r];
+                    z2 y = j > c ? Cb[j] : Lb[at(c, j)], u = Lb[at(r, j)];
+                    if (j > c) y = zconj(y);
+                    if (j == c) u = zmk(0.0, 0.0);
+                    zmsub(u, l, y);
+                    Lb[at(r, j)] = u;
+                }
+            }
+    }
+}
+
+// X_b = L_b^{-1} of A_b = L_b L_b^H (packed lower in sL, in place) for the blocks
+// of a chunk, by 8 x 8 blocks: left-looking, one warp per block of
+//   T_IJ = A_IJ - sum_{K<J} L_IK L_JK^H,  X_JJ from T_JJ (chol_inv8),
+//   L_IJ = T_IJ X_JJ^H,  U_JK = sum_{K<=M<J} L_JM X_MK,  X_JK = -X_JJ U_JK,
+// so that every block is rounded once per formula.  X_JK takes the place of
+// L_JK one step after U_JK has read row J of L.  Ends with __syncthreads().
+template <int MT, bool FULL>
+__device__ __forceinline__ void inverse_chunk(const LevelArgs &a, int64_t t0, z2 *sL, z2 *sC, z2 *sU, int nbh) {
+    const int m = FULL ? MT : a.m;
+    if constexpr (MT == 8) {
+        chol_inv8<MT>(a, t0, sL, sC, nbh, 0, m);
+        return;
+    } else {
+        constexpr int SL = Split64<MT>::SL, SU = Split64<MT>::SU, KS = MT / 8;
+        const z2 zero = zmk(0.0, 0.0);
+        const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, tq = lane & 3, warp = tid >> 5, nw = blockDim.x >> 5;
+        const int g8 = FULL ? KS : (m + 7) >> 3;
+        for (int J = 0; J <= g8; ++J) {
+            // T_IJ for I >= J, and row J - 1 of X (J - 1 blocks)
+            const int nT = J > 0 ? g8 - J : 0, nX = J > 1 ? J - 1 : 0, n1 = nT + nX;
+            for (int e = warp; e < nbh * n1; e += nw) {
+                const int b = e / n1, f = e - b * n1;
+                z2 *Lb = sL + b * SL;
+                z2 v[2];
+                int ex[2];
+                if (f < nT) {
+                    const int I = J + f;
+                    auto row = [&](int r, int k) { return (FULL || r < m) ? Lb[tri(r, k)] : zero; };
+                    split_tile<kConjB, false, KS>(J, [&](int i, int k) { return row(8 * I + i, k); },
+                                                  [&](int i, int k) { return row(8 * J + i, k); }, I == J, v, ex);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const int r = 8 * I + g, c = 8 * J + 2 * tq + j;
+                        if ((!FULL && r >= m) || c > r) continue;
+                        z2 &u = Lb[tri(r, c)];
+                        const double sc = -split_scale(ex[j]);
+                        u.x = fma(v[j].x, sc, u.x);
+                        u.y = r == c ? 0.0 : fma(v[j].y, sc, u.y);
+                    }
+                } else {
+                    const int I = J - 1, K = f - nT;
+                    const z2 *Ub = sU + b * SU + 8 * K;
+                    auto x = [&](int i, int k) { return (k <= i && (FULL || 8 * I + i < m)) ? Lb[tri(8 * I + i, 8 * I + k)] : zero; };
+                    split_tile<kPlain, true, 1>(1, [&](int i, int k) { return (FULL || 8 * I + k < m) ? Ub[k * MT + i] : zero; }, x, false, v, ex);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const int r = 8 * I + 2 * tq + j;
+                        if (FULL || r < m)
+                            Lb[tri(r, 8 * K + g)] = zmk(dneg_bits(split_scaled(v[j].x, ex[j])), dneg_bits(split_scaled(v[j].y, ex[j])));
+                    }
+                }
+            }
+            if (J == g8) break;
+            __syncthreads();
+            chol_inv8<MT>(a, t0, sL, sC, nbh, 8 * J, min(8, m - 8 * J));
+            // L_IJ for I > J, and U_JK for K < J
+            const int nL = g8 - 1 - J, n2 = nL + J;
+            for (int e = warp; e < nbh * n2; e += nw) {
+                const int b = e / n2, f = e - b * n2;
+                z2 *Lb = sL + b * SL;
+                z2 v[2];
+                int ex[2];
+                if (f < nL) {
+                    const int I = J + 1 + f;
+                    // block column J is complete (8 wide) as there is a row below it
+                    split_tile<kConjB, true, 1>(1, [&](int i, int k) { return (FULL || 8 * I + i < m) ? Lb[tri(8 * I + i, 8 * J + k)] : zero; },
+                                                [&](int i, int k) { return k <= i ? Lb[tri(8 * J + i, 8 * J + k)] : zero; }, false, v, ex);
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+                        if (FULL || 8 * I + g < m)
+                            Lb[tri(8 * I + g, 8 * J + 2 * tq + j)] = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
+                } else {
+                    const int K = f - nL;
+                    split_tile<kPlain, false, KS>(
+                        J - K,
+                        [&](int i, int k) {     // column i of X
+                            const int r = 8 * K + k, c = 8 * K + i;
+                            return c <= r ? Lb[tri(r, c)] : zero;
+                        },
+                        [&](int i, int k) { return (FULL || 8 * J + i < m) ? Lb[tri(8 * J + i, 8 * K + k)] : zero; }, false, v, ex);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+                        if (FULL || 8 * J + 2 * tq + j < m)
+                            sU[b * SU + (2 * tq + j) * MT + 8 * K + g] = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
+                }
+            }
+            __syncthreads();
+        }
+        __syncthreads();
+    }
+}
+
+// One chunk of nb odd blocks of a factor level (see factor_chunk).
+template <int MT, bool FULL>
+__device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, unsigned char *smem_raw) {
+    constexpr int LDZ = Split64<MT>::LDZ, SL = Split64<MT>::SL, KS = MT / 8;
+    const int m = FULL ? MT : a.m, nb = a.nb, NT = blockDim.x, tid = threadIdx.x;
+    const int mm = m * m, m2 = 2 * m;
+    const int64_t t0 = chunk * nb;
+    const int nbh = (int)min((int64_t)nb, a.no - t0);
+    z2 *sL = reinterpret_cast<z2 *>(smem_raw);              // [nb][SL] A_2t, then X, then P^H P
+    z2 *sZ = sL + (size_t)nb * SL;                            // [nb][MT][LDZ] [B_l | B_r^H], then Z = [P | Q]
+    z2 *sC = sZ + (size_t)nb * MT * LDZ;                      // [nb][SC]
+    z2 *sU = sC + (size_t)nb * Split64<MT>::SC;               // [nb][SU]
+    const z2 zero = zmk(0.0, 0.0);
+
+    for (int e = tid; e < nbh * mm; e += NT) {
+        const int b = e / mm, rem = e - b * mm, r = rem / m, c = rem - r * m;
+        const int64_t pos = 2 * (t0 + b);
+        if (r >= c) sL[b * SL + tri(r, c)] = CRS_IN(a, kDbgA, pos * mm + rem) ? a.A[pos * mm + rem] : zero;
+        sZ[(b * MT + r) * LDZ + c] = (pos >= 1 && CRS_IN(a, kDbgB, (pos - 1) * mm + rem)) ? a.B[(pos - 1) * mm + rem] : zero;
+        sZ[(b * MT + c) * LDZ + m + r] =
+            (pos + 1 < a.Nl && CRS_IN(a, kDbgB, pos * mm + rem)) ? zconj(a.B[pos * mm + rem]) : zero;
+    }
+    __syncthreads();
+    inverse_chunk<MT, FULL>(a, t0, sL, sC, sU, nbh);
+
+    const int lane = tid & 31, g = lane >> 2, tq = lane & 3, warp = tid >> 5, nw = NT >> 5;
+    const int g8 = (FULL || KS == 1) ? KS : (m + 7) >> 3, ngrp = 2 * g8;
+    z2 *sW = sL;    // P^H P
+
+    // Z = X [B_l | B_r^H] of 8 columns of a block in place, by one warp, the rows
+    // from the bottom up.  Column groups 0 .. g8-1 are P, the others Q.
+    auto z_task = [&](int b, int cg) {
+        const int64_t t = t0 + b;
+        const bool inP = cg < g8;
+        const int c0 = 8 * (inP ? cg : cg - g8), nc = m - c0, col = (inP ? c0 : m + c0) + g;
+        z2 *Zb = sZ + b * MT * LDZ;
+        const z2 *Xb = sL + b * SL;
+        if (inP ? t >= 1 : 2 * t + 1 < a.Nl) {
+            for (int R = g8 - 1; R >= 0; --R) {
+                z2 v[2];
+                int ex[2];
+                split_tile<kPlain, true, KS>(
+                    R + 1, [&](int i, int k) { return (FULL || (i < nc && k < m)) ? Zb[k * LDZ + col - g + i] : zero; },
+                    [&](int i, int k) { return ((FULL || 8 * R + i < m) && k <= 8 * R + i) ? Xb[tri(8 * R + i, k)] : zero; }, false, v, ex);
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int r = 8 * R + 2 * tq + j;
+                    if (FULL || (g < nc && r < m))
+                        Zb[r * LDZ + col] = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
+                }
+                __syncwarp();
+            }
+        }
+        // (a zero coupling leaves its half of Z zero)
+        if (FULL || g < nc)
+            for (int r = tq; r < m; r += 4) {
+                const int64_t o = t * 2 * (int64_t)mm + r * m2 + col;
+                if (CRS_IN(a, kDbgZ, o)) a.Z[o] = Zb[r * LDZ + col];
+            }
+    };
+
+    // Entry (p, q), q <= p, of P^H P of block b: kept in sW for the left even block,
+    // or for the chunk's first block given to the previous chunk.
+    auto put_pp = [&](int b, int p, int q, z2 w) {
+        const int64_t t = t0 + b;
+        if (b > 0) {
+            sW[b * SL + tri(p, q)] = w;
+        } else if (a.inline_fix) {
+            // the previous chunk (same CTA, earlier) left V = A - Q^H Q
+            const int64_t o = (t - 1) * mm;
+            if (CRS_IN(a, kDbgAn, o + p * m + q) && CRS_IN(a, kDbgAn, o + q * m + p)) {
+                z2 u = zsub(a.An[o + p * m + q], w);
+                if (p == q) u.y = 0.0;
+                a.An[o + p * m + q] = u;
+                if (p != q) a.An[o + q * m + p] = zconj(u);
+            }
+        } else if (CRS_IN(a, kDbgWbd, chunk * mm + p * m + q)) {
+            a.Wbd[chunk * mm + p * m + q] = w;
+        }
+    };
+    // Entry (p, q) of Q^H P = -F, the next level's B.
+    auto put_qp = [&](int b, int p, int q, z2 w) {
+        const int64_t o = (t0 + b - 1) * mm + p * m + q;
+        if (CRS_IN(a, kDbgBn, o)) a.Bn[o] = zneg(w);
+    };
+    // A - Q^H Q at entry (p, q), q <= p, of block b's right even block
+    auto sub_qq = [&](int b, int p, int q, z2 v, int ex) {
+        const int64_t oa = (2 * (t0 + b) + 1) * mm + p * m + q;
+        z2 u = CRS_IN(a, kDbgA, oa) ? a.A[oa] : zero;
+        const double sc = -split_scale(ex);
+        u.x = fma(v.x, sc, u.x);
+        u.y = p == q ? 0.0 : fma(v.y, sc, u.y);
+        return u;
+    };
+    // ... complete unless the right neighbour is in the next chunk
+    auto put_v = [&](int b, int p, int q, z2 u) {
+        const int64_t o = (t0 + b) * mm;
+        if (b + 1 < nbh) u = zsub(u, sW[(b + 1) * SL + tri(p, q)]);
+        if (CRS_IN(a, kDbgAn, o + p * m + q)) a.An[o + p * m + q] = u;
+        if (p != q && CRS_IN(a, kDbgAn, o + q * m + p)) a.An[o + q * m + p] = zconj(u);
+    };
+
+    // Z^H Z by tiles (row group I >= column group J): pass 0 has P^H P and Q^H P,
+    // pass 1 Q^H Q.
+    const int ntri = g8 * (g8 + 1) / 2;
+    auto h_task = [&](int b, int pass, int f) {
+        const int64_t t = t0 + b;
+        int I, J;
+        const bool pJ = pass == 0, pI = pass == 0 && f < ntri;
+        if (pI || !pJ) {
+            I = tri_row(f);
+            J = f - I * (I + 1) / 2;
+        } else {
+            I = (f - ntri) / g8;
+            J = f - ntri - I * g8;
+        }
+        if ((pJ && t < 1) || (!pI && 2 * t + 1 >= a.Nl)) return;
+        const z2 *Zb = sZ + b * MT * LDZ;
+        const z2 *zi = Zb + 8 * I + (pI ? 0 : m), *zj = Zb + 8 * J + (pJ ? 0 : m);
+        const int ni = m - 8 * I, nj = m - 8 * J;
+        z2 v[2];
+        int ex[2];
+        split_tile<kConjA, false, KS>(
+            g8, [&](int i, int k) { return (FULL || (i < ni && k < m)) ? zi[k * LDZ + i] : zero; },
+            [&](int i, int k) { return (FULL || (i < nj && k < m)) ? zj[k * LDZ + i] : zero; }, zi == zj, v, ex);
+        const int p = 8 * I + g;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int q = 8 * J + 2 * tq + j;
+            if (!FULL && (p >= m || q >= m)) continue;
+            if (!pJ) {
+                if (q <= p) put_v(b, p, q, sub_qq(b, p, q, v[j], ex[j]));
+                continue;
+            }
+            z2 w = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
+            if (!pI) {
+                put_qp(b, p, q, w);
+            } else if (q <= p) {
+                if (p == q) w.y = 0.0;
+                put_pp(b, p, q, w);
+            }
+        }
+    };
+
+    if constexpr (MT == 8) {
+        // Blocks that fill at least half of the warps: one warp takes a block
+        // through all five products, Z staying in registers (an entry of Z is
+        // in the lane that needs it for Z^H Z, and X, P and Q are cut once).
+        // Halves the integer work per block against the tasks below, which
+        // spread a block over warps; the same numbers.
+        if (2 * nbh > nw) {
+            for (int b = warp; b < nbh; b += nw) {
+                const int64_t t = t0 + b;
+                const bool hasL = t >= 1, hasR = 2 * t + 1 < a.Nl;
+                z2 *Zb = sZ + b * MT * LDZ;
+                const z2 *Xb = sL + b * SL;
+                z2 x[2], z[2][2];
+                SplitCut cx, cz[2];
+                SplitJoint jt[2];
+                unsigned mx[2], mz[2];
+                bool ok = true;
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int k = 2 * tq + j;
+                    x[j] = ((FULL || g < m) && k <= g) ? Xb[tri(g, k)] : zero;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) z[h][j] = (FULL || (g < m && k < m)) ? Zb[k * LDZ + (h ? m : 0) + g] : zero;
+                    const int64_t o = t * mm + g * m + k;
+                    if ((FULL || (g < m && k < m)) && CRS_IN(a, kDbgL, o)) a.L[o] = x[j];
+                }
+                split_joint_exp(x[0], x[1], mx[0], mx[1]);
+                const int c0 = split_exp(mx[0]), c1 = split_exp(mx[1]);
+                split_cut(cx, x[0], x[1], c0, c1);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    jt[h].term(split_mag(z[h][0]), mx[0]);
+                    jt[h].term(split_mag(z[h][1]), mx[1]);
+                    if (jt[h].finish() || jt[h].ea < kSplitSumTiny) ok = false;
+                    split_cut(cz[h], z[h][0], z[h][1], jt[h].ea - c0, jt[h].ea - c1);
+                    SplitAcc acc;
+                    split_start(acc, kSplitStart);
+                    split_mma<kPlain>(cz[h], cx, acc);
+                    double v[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        int sum[kSplitDigits];
+#pragma unroll
+                        for (int d = 0; d < kSplitDigits; ++d) sum[d] = __float_as_int(acc[d][j]);
+                        v[j] = split_scaled(split_value<true>(sum), jt[h].ea);
+                    }
+                    z[h][0] = zmk(v[0], v[2]);
+                    z[h][1] = zmk(v[1], v[3]);
+                    mz[h] = split_max4(max(split_mag(z[h][0]), split_mag(z[h][1])));
+                    if (split_unsafe(mz[h])) ok = false;
+                }
+                const int ez[2] = {split_exp(mz[0]), split_exp(mz[1])};
+                if (2 * min(ez[0], ez[1]) < kSplitSumTiny) ok = false;
+                ok = __all_sync(0xffffffffu, ok);
+                if (lane == 0) sC[b * Split64<MT>::SC].x = ok ? 1.0 : 0.0;
+                __syncwarp();
+                if (!ok) {      // out of the split's range somewhere
+                    z_task(b, 0);
+                    z_task(b, 1);
+                    __syncwarp();
+                    h_task(b, 0, 0);
+                    h_task(b, 0, 1);
+                    continue;
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const int r = 2 * tq + j;
+                        const int64_t o = t * 2 * (int64_t)mm + r * m2 + (h ? m : 0) + g;
+                        if ((FULL || (g < m && r < m)) && CRS_IN(a, kDbgZ, o)) a.Z[o] = z[h][j];
+                    }
+                    split_cut(cz[h], z[h][0], z[h][1], ez[h], ez[h]);
+                }
+                // P^H P, Q^H P, Q^H Q
+#pragma unroll
+                for (int f = 0; f < 3; ++f) {
+                    const int hi = f > 0, hj = f > 1;
+                    if ((!hj && !hasL) || (hi && !hasR)) continue;
+                    SplitAcc acc;
+                    split_start(acc, kSplitStart);
+                    split_mma<kConjA>(cz[hi], cz[hj], acc);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const int p = g, q = 2 * tq + j, ex = ez[hi] + __shfl_sync(0xffffffffu, ez[hj], 8 * tq + 4 * j);
+                        int s0[kSplitDigits], s1[kSplitDigits];
+#pragma unroll
+                        for (int d = 0; d < kSplitDigits; ++d) {
+                            s0[d] = __float_as_int(acc[d][j]);
+                            s1[d] = __float_as_int(acc[d][j + 2]);
+                        }
+                        const z2 v = zmk(split_value<true>(s0), split_value<true>(s1));
+                        if ((!FULL && (p >= m || q >= m)) || (f != 1 && q > p)) continue;
+                        if (f == 2) {
+                            Zb[p * LDZ + q] = sub_qq(b, p, q, v, ex);
+                        } else {
+                            z2 w = zmk(split_scaled(v.x, ex), split_scaled(v.y, ex));
+                            if (f == 1) {
+                                put_qp(b, p, q, w);
+                            } else {
+                                if (p == q) w.y = 0.0;
+                                put_pp(b, p, q, w);
+                            }
+                        }
+                    }
+                }
+            }
+            __syncthreads();
+            for (int b = warp; b < nbh; b += nw) {
+                if (2 * (t0 + b) + 1 >= a.Nl) continue;
+                if (sC[b * Split64<MT>::SC].x == 0.0) {
+                    h_task(b, 1, 0);
+                    continue;
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int p = g, q = 2 * tq + j;
+                    if ((FULL || p < m) && q <= p) put_v(b, p, q, sZ[(b * MT + p) * LDZ + q]);
+                }
+            }
+            __syncthreads();
+        }
+    }
+    if (MT > 8 || 2 * nbh <= nw) {
+        for (int e = warp; e < nbh * ngrp; e += nw) z_task(e / ngrp, e % ngrp);
+        // keep X
+        for (int e = tid; e < nbh * mm; e += NT) {
+            const int b = e / mm, rem = e - b * mm, r = rem / m, c = rem - r * m;
+            if (CRS_IN(a, kDbgL, (t0 + b) * mm + rem)) a.L[(t0 + b) * mm + rem] = r >= c ? sL[b * SL + tri(r, c)] : zero;
+        }
+        __syncthreads();
+        for (int pass = 0; pass < 2; ++pass) {
+            const int nt = pass == 0 ? ntri + g8 * g8 : ntri;
+            for (int e = warp; e < nbh * nt; e += nw) h_task(e / nt, pass, e % nt);
+            __syncthreads();
+        }
+    }
+    if (a.bd_count) {
+        const int nl = m * (m + 1) / 2;
+        const int sec = bd_arrive(a.bd_count, chunk, crs_num_ctas(a.no, a.nb));
+        for (int e = tid; e < ((sec & 1) ? nl : 0); e += NT) factor_fix_entry<double, true>(a, chunk, e);
+        for (int e = tid; e < ((sec & 2) ? nl : 0); e += NT) factor_fix_entry<double, true>(a, chunk + 1, e);
+    }
+}
+
+// One chunk of nb odd blocks and right-hand-side columns [cchunk*kc, +kc) of
+// a down-sweep level: r = X y_odd, then P^H r, then v = (y_even - Q^H r) - P^H r.
+// One warp per block, 8 rows and 8 columns.
+template <int MT, bool FULL>
+__device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chunk, int cchunk,
+                                                       unsigned char *smem_raw) {
+    constexpr int KS = MT / 8;
+    const int m = FULL ? MT : a.m, k = a.k, nb = a.nb, kc = a.kc, NT = blockDim.x, tid = threadIdx.x;
+    const int mm = m * m, m2 = 2 * m, mk = m * k;
+    const int cb = cchunk * kc, kw = min(kc, k - cb);
+    const int64_t t0 = chunk * nb;
+    const int nbh = (int)min((int64_t)nb, a.no - t0);
+    z2 *sR = reinterpret_cast<z2 *>(smem_raw);              // [nb][MT][kc] r of odd t0 + b
+    z2 *sW = sR + (size_t)nb * MT * kc;                       // [nb][MT][kc] P^H r of odd t0 + b
+    const z2 zero = zmk(0.0, 0.0);
+    const int lane = tid & 31, g = lane >> 2, tq = lane & 3, warp = tid >> 5, nw = NT >> 5;
+    const int g8 = (FULL || KS == 1) ? KS : (m + 7) >> 3, ncg = (kw + 7) >> 3, per = g8 * ncg;
+
+    for (int e = warp; e < nbh * per; e += nw) {
+        const int b = e / per, rem = e - b * per, R = rem / ncg, n0 = 8 * (rem - R * ncg);
+        const int64_t t = t0 + b, yo = 2 * t * mk + cb + n0, xo = t * mm + 8 * R * m;
+        const int nc = kw - n0;
+        z2 v[2];
+        int ex[2];
+        split_tile<kPlain, true, KS>(
+            R + 1, [&](int i, int s) { return (i < nc && (FULL || s < m) && CRS_IN(a, kDbgY, yo + s * k + i)) ? __ldg(a.y + yo + s * k + i) : zero; },
+            [&](int i, int s) {
+                return ((FULL || 8 * R + i < m) && s <= 8 * R + i && CRS_IN(a, kDbgL, xo + i * m + s)) ? __ldg(a.L + xo + i * m + s) : zero;
+            },
+            false, v, ex);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int r = 8 * R + 2 * tq + j;
+            if (g >= nc || (!FULL && r >= m)) continue;
+            const z2 w = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
+            sR[(b * MT + r) * kc + n0 + g] = w;
+            const int64_t o = t * mk + r * k + cb + n0 + g;
+            if (CRS_IN(a, kDbgR, o)) a.r[o] = w;
+        }
+    }
+    __syncthreads();
+    for (int pass = 0; pass < 2; ++pass) {      // 0: P^H r, 1: Q^H r
+        for (int e = warp; e < nbh * per; e += nw) {
+            const int b = e / per, rem = e - b * per, G = rem / ncg, n0 = 8 * (rem - G * ncg);
+            const int64_t t = t0 + b, zo = t * m2 * m + (pass ? m : 0) + 8 * G;
+            if (pass ? 2 * t + 1 >= a.Nl : t < 1) continue;
+            const int nc = kw - n0, np = m - 8 * G;
+            const z2 *Rb = sR + b * MT * kc + n0;
+            z2 v[2];
+            int ex[2];
+            split_tile<kConjA, false, KS>(
+                g8,
+                [&](int i, int s) { return ((FULL || (i < np && s < m)) && CRS_IN(a, kDbgZ, zo + s * m2 + i)) ? __ldg(a.Z + zo + s * m2 + i) : zero; },
+                [&](int i, int s) { return (i < nc && (FULL || s < m)) ? Rb[s * kc + i] : zero; }, false, v, ex);
+            const int p = 8 * G + g;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int n = 2 * tq + j;
+                if ((!FULL && p >= m) || n >= nc) continue;
+                const int64_t rem2 = (int64_t)p * k + cb + n0 + n;
+                if (pass == 0) {
+                    const z2 w = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
+                    if (b > 0) {
+                        sW[(b * MT + p) * kc + n0 + n] = w;
+                    } else if (a.inline_fix) {
+                        const int64_t o = (t - 1) * mk + rem2;
+                        if (CRS_IN(a, kDbgYn, o)) a.yn[o] = zsub(a.yn[o], w);
+                    } else if (CRS_IN(a, kDbgCbd, chunk * mk + rem2)) {
+                        a.cbd[chunk * mk + rem2] = w;
+                    }
+                } else {
+                    const int64_t oy = (2 * t + 1) * mk + rem2;
+                    z2 u = CRS_IN(a, kDbgY, oy) ? __ldg(a.y + oy) : zero;
+                    const double sc = -split_scale(ex[j]);
+                    u.x = fma(v[j].x, sc, u.x);
+                    u.y = fma(v[j].y, sc, u.y);
+                    if (b + 1 < nbh) u = zsub(u, sW[((b + 1) * MT + p) * kc + n0 + n]);
+                    if (CRS_IN(a, kDbgYn, t * mk + rem2)) a.yn[t * mk + rem2] = u;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    if (a.bd_count) {
+        // counters of this right-hand-side chunk: [cchunk][boundary]
+        const int64_t ncta = crs_num_ctas(a.no, a.nb);
+        const int sec = bd_arrive(a.bd_count + cchunk * ncta, chunk, ncta);
+        for (int e = tid; e < ((sec & 1) ? m * kw : 0); e += NT)
+            solve_down_fix_entry<double, true>(a, chunk, (e / kw) * k + cb + e % kw);
+        for (int e = tid; e < ((sec & 2) ? m * kw : 0); e += NT)
+            solve_down_fix_entry<double, true>(a, chunk + 1, (e / kw) * k + cb + e % kw);
+    }
+}
+
+// One chunk of an up-sweep level: w = r - Z [x_left; x_right], x_odd = X^H w; the
+// even unknowns are copied.
+template <int MT, bool FULL>
+__device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk, int cchunk,
+                                                     unsigned char *smem_raw) {
+    constexpr int KS = MT / 8;
+    const int m = FULL ? MT : a.m, k = a.k, nb = a.nb, kc = a.kc, NT = blockDim.x, tid = threadIdx.x;
+    const int mm = m * m, m2 = 2 * m, mk = m * k;
+    const int cb = cchunk * kc, kw = min(kc, k - cb);
+    const int64_t t0 = chunk * nb;
+    const int nbh = (int)min((int64_t)nb, a.no - t0);
+    z2 *sW = reinterpret_cast<z2 *>(smem_raw);              // [nb][MT][kc]
+    const z2 zero = zmk(0.0, 0.0);
+    const int lane = tid & 31, g = lane >> 2, tq = lane & 3, warp = tid >> 5, nw = NT >> 5;
+    const int g8 = (FULL || KS == 1) ? KS : (m + 7) >> 3, ncg = (kw + 7) >> 3, per = g8 * ncg;
+
+    const bool failed = a.level == 0 && *a.status != CRS_NO_FAIL;   // the result is NaN
+    for (int e = tid; e < nbh * m * kw; e += NT) {
+        const int b = e / (m * kw), rem = e - b * (m * kw), r = rem / kw, c = rem - r * kw;
+        const int64_t t = t0 + b, o = (int64_t)r * k + cb + c;
+        if (failed && CRS_IN(a, kDbgX, 2 * t * mk + o)) a.x[2 * t * mk + o] = zmk(qnan(0.0), qnan(0.0));
+        if (t < a.ne && CRS_IN(a, kDbgX, (2 * t + 1) * mk + o))
+            a.x[(2 * t + 1) * mk + o] =
+                failed ? zmk(qnan(0.0), qnan(0.0)) : (CRS_IN(a, kDbgXn, t * mk + o) ? __ldg(a.xn + t * mk + o) : zero);
+    }
+    if (failed) return;
+
+    for (int e = warp; e < nbh * per; e += nw) {
+        const int b = e / per, rem = e - b * per, R = rem / ncg, n0 = 8 * (rem - R * ncg);
+        const int64_t t = t0 + b, zo = t * m2 * m + 8 * R * m2;
+        const int nc = kw - n0;
+        const bool hasL = t >= 1, hasR = t < a.ne;
+        z2 v[2];
+        int ex[2];
+        // terms 0 .. 8 g8 - 1: P and x_left, 8 g8 .. : Q and x_right
+        split_tile<kPlain, true, 2 * KS>(
+            2 * g8,
+            [&](int i, int s) {
+                const bool right = s >= 8 * g8;
+                const int q = right ? s - 8 * g8 : s;
+                const int64_t o = (right ? t : t - 1) * mk + q * k + cb + n0 + i;
+                return (i < nc && (FULL || q < m) && (right ? hasR : hasL) && CRS_IN(a, kDbgXn, o)) ? __ldg(a.xn + o) : zero;
+            },
+            [&](int i, int s) {
+                const bool right = s >= 8 * g8;
+                const int q = right ? s - 8 * g8 : s;
+                const int64_t o = zo + i * m2 + (right ? m : 0) + q;
+                return ((FULL || (8 * R + i < m && q < m)) && CRS_IN(a, kDbgZ, o)) ? __ldg(a.Z + o) : zero;
+            },
+            false, v, ex);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int r = 8 * R + 2 * tq + j;
+            const int64_t o = t * mk + r * k + cb + n0 + g;
+            if (g >= nc || (!FULL && r >= m) || !CRS_IN(a, kDbgR, o)) continue;
+            z2 w = __ldg(a.r + o);
+            const double sc = -split_scale(ex[j]);
+            w.x = fma(v[j].x, sc, w.x);
+            w.y = fma(v[j].y, sc, w.y);
+            sW[(b * MT + r) * kc + n0 + g] = w;
+        }
+    }
+    __syncthreads();
+    for (int e = warp; e < nbh * per; e += nw) {
+        const int b = e / per, rem = e - b * per, G = rem / ncg, n0 = 8 * (rem - G * ncg);
+        const int64_t t = t0 + b, xo = t * mm + 8 * G * m + 8 * G;
+        const int nc = kw - n0, np = m - 8 * G;
+        const z2 *Wb = sW + (b * MT + 8 * G) * kc + n0;
+        z2 v[2];
+        int ex[2];
+        // X[s][p] is zero for s < p: terms from row 8 G on
+        split_tile<kConjA, false, KS>(
+            g8 - G, [&](int i, int s) { return ((FULL || (i < np && s < np)) && i <= s && CRS_IN(a, kDbgL, xo + s * m + i)) ? __ldg(a.L + xo + s * m + i) : zero; },
+            [&](int i, int s) { return (i < nc && (FULL || s < np)) ? Wb[s * kc + i] : zero; }, false, v, ex);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int p = 8 * G + g, n = 2 * tq + j;
+            const int64_t o = 2 * t * mk + (int64_t)p * k + cb + n0 + n;
+            if ((FULL || p < m) && n < nc && CRS_IN(a, kDbgX, o))
+                a.x[o] = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
+        }
+    }
+}
+
+}  // namespace crs

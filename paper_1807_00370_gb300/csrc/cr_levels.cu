@@ -1,6 +1,8 @@
 // cr_levels.cu -- the per-level kernels of classic cyclic reduction in FP64
 // (one chunk of odd blocks per CTA; the steps themselves are in cr_core.cuh)
 // and their host-side launchers.
+#include <algorithm>
+
 #include "cr_launch.h"
 #include "cr_core.cuh"
 
@@ -41,7 +43,7 @@ __global__ void __launch_bounds__(256) k_solve_up(LevelArgsT<R> a) {
     solve_up_chunk<MT, R>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
 
-// The FP64 sweeps of class 16 at the default 128 threads, with registers
+// The FMA sweeps of class 16 at the default 128 threads, with registers
 // capped so that five CTAs fit on an SM (16 warps otherwise): more warps to
 // cover the loads at the start of each chunk.
 __global__ void __launch_bounds__(128, 5) k_solve_down_odd_16c(LevelArgsT<double> a) {
@@ -71,6 +73,23 @@ template <int MT, class R>
 __global__ void __launch_bounds__(256) k_solve_up_wide(LevelArgsT<R> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_up_chunk<MT, R, true>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
+}
+
+// The split forms of the FP64 levels (cr_core64.cuh).
+template <int MT>
+__global__ void __launch_bounds__(256) k_factor_split(LevelArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    factor_chunk_split<MT>(a, a.c_begin + blockIdx.x, smem_raw);
+}
+template <int MT>
+__global__ void __launch_bounds__(256) k_solve_down_split(LevelArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    solve_down_chunk_split<MT>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
+}
+template <int MT>
+__global__ void __launch_bounds__(256) k_solve_up_split(LevelArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    solve_up_chunk_split<MT>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
 
 // ------------------------------------------------------------------ adjoint
@@ -126,10 +145,10 @@ __global__ void k_nan_if_failed(z2 *x, int64_t n, const unsigned long long *stat
 // N = 2^14, m = 64, k = 32); crsolve_tile_set overrides them.
 static TileShape g_tiles[5] = {
     {32, 32, 32, 256, 256},  // MT = 4
-    {16, 16, 16, 256, 256},  // MT = 8
+    {16, 16, 16, 256, 128},  // MT = 8
     {8, 4, 8, 256, 128},     // MT = 16
-    {2, 1, 16, 256, 256},    // MT = 32
-    {1, 1, 16, 256, 256},    // MT = 64
+    {2, 1, 8, 256, 128},     // MT = 32
+    {1, 1, 8, 256, 128},     // MT = 64
 };
 
 static int mt_slot(int mt) {
@@ -199,8 +218,10 @@ int pick_mt(int m) {
     return 0;
 }
 
-// Per block: packed L (later P^H P) and packed V, Z = [P | Q], 1/diag(L);
-// rsize = bytes of the real type (8 for FP64, 4 for FP32).
+// Shared memory that a tile shape is accepted by (and that the batched kernel
+// takes): per block packed L (later P^H P) and packed V, Z = [P | Q], 1/diag(L), or
+// the split form's layout where that is larger; rsize = bytes of the real type
+// (8 for FP64, 4 for FP32).
 size_t factor_smem_bytes(int mt, int nb, int rsize) {
     const size_t tri = (size_t)mt * (mt + 1) / 2, cs = 2 * (size_t)rsize;
     size_t b = (size_t)nb * ((2 * tri + 2 * (size_t)mt * mt) * cs + (size_t)mt * rsize);
@@ -208,6 +229,7 @@ size_t factor_smem_bytes(int mt, int nb, int rsize) {
         b += 1024 + tc_stage_bytes(mt);                 // tensor-core operand stages (1 KB aligned)
         b += (size_t)nb * mt * kF32LdE * cs;             // L^{-1} of every block (padded rows)
     }
+    if (rsize == 8 && mt >= 8) b = std::max(b, nb * factor64_entries(mt) * cs);
     return b;
 }
 
@@ -224,31 +246,31 @@ size_t solve_smem_bytes(int mt, int nb, int kc, int panels, int rsize) {
 // tile shape that set_tile_shape accepted can launch.
 template <int MT, class R>
 static cudaError_t prepare_mt_r(int smem_optin) {
-    cudaError_t e;
-    e = cudaFuncSetAttribute(k_factor_odd<MT, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
-    if (e != cudaSuccess) return e;
-    if constexpr (MT == 64 && sizeof(R) == 4) {
-        e = cudaFuncSetAttribute(k_factor_odd_f32_64, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
-        if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    auto allow = [&](auto *kernel) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
+    };
+    if constexpr (Forms<MT, R>::split) {
+        allow(k_factor_split<MT>);
+        allow(k_solve_down_split<MT>);
+        allow(k_solve_up_split<MT>);
     }
-    if constexpr (MT == 16 && sizeof(R) == 8) {
-        e = cudaFuncSetAttribute(k_solve_down_odd_16c, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k_solve_up_16c, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
-        if (e != cudaSuccess) return e;
+    if constexpr (Forms<MT, R>::fma) {
+        allow(k_factor_odd<MT, R>);
+        if constexpr (MT == 64 && sizeof(R) == 4) allow(k_factor_odd_f32_64);
+        if constexpr (MT < 32) {
+            allow(k_factor_odd_wide<MT, R>);
+            allow(k_solve_down_odd_wide<MT, R>);
+            allow(k_solve_up_wide<MT, R>);
+        }
+        allow(k_solve_down_odd<MT, R>);
+        allow(k_solve_up<MT, R>);
+        if constexpr (MT == 16 && sizeof(R) == 8) {
+            allow(k_solve_down_odd_16c);
+            allow(k_solve_up_16c);
+        }
     }
-    if constexpr (MT < 32) {
-        e = cudaFuncSetAttribute(k_factor_odd_wide<MT, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k_solve_down_odd_wide<MT, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 smem_optin);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k_solve_up_wide<MT, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
-        if (e != cudaSuccess) return e;
-    }
-    e = cudaFuncSetAttribute(k_solve_down_odd<MT, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_solve_up<MT, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
+    return e;
 }
 
 template <int MT>
@@ -355,15 +377,22 @@ template <int MT, class R>
 static cudaError_t factor_odd_mt(const LevelArgsT<R> &a, cudaStream_t s) {
     const unsigned grid = odd_grid(a);
     const int th = sizeof(R) == 4 ? tile_shape32(MT).threads : tile_shape(MT).threads;
-    if constexpr (MT == 64 && sizeof(R) == 4) {
-        k_factor_odd_f32_64<<<grid, th, factor_smem_bytes(MT, a.nb, sizeof(R)), s>>>(a);
-    } else if constexpr (MT < 32) {
-        if (factor_wide<MT, R>(a))
-            k_factor_odd_wide<MT, R><<<grid, th, factor_smem_bytes(MT, a.nb, sizeof(R)), s>>>(a);
-        else
-            k_factor_odd<MT, R><<<grid, th, factor_smem_bytes(MT, a.nb, sizeof(R)), s>>>(a);
-    } else {
-        k_factor_odd<MT, R><<<grid, th, factor_smem_bytes(MT, a.nb, sizeof(R)), s>>>(a);
+    if constexpr (Forms<MT, R>::split) {
+        if (split_form(a.m, sizeof(R))) {
+            k_factor_split<MT><<<grid, th, a.nb * factor64_entries(MT) * sizeof(z2), s>>>(a);
+            return cudaGetLastError();
+        }
+    }
+    if constexpr (Forms<MT, R>::fma) {
+        const size_t smem = factor_smem_bytes(MT, a.nb, sizeof(R));
+        if constexpr (MT == 64 && sizeof(R) == 4) {
+            k_factor_odd_f32_64<<<grid, th, smem, s>>>(a);
+        } else if constexpr (MT < 32) {
+            if (factor_wide<MT, R>(a)) k_factor_odd_wide<MT, R><<<grid, th, smem, s>>>(a);
+            else k_factor_odd<MT, R><<<grid, th, smem, s>>>(a);
+        } else {
+            k_factor_odd<MT, R><<<grid, th, smem, s>>>(a);
+        }
     }
     return cudaGetLastError();
 }
@@ -372,19 +401,29 @@ template <int MT, class R>
 static cudaError_t solve_down_odd_mt(const LevelArgsT<R> &a, cudaStream_t s) {
     const dim3 grid(odd_grid(a), (unsigned)((a.k + a.kc - 1) / a.kc));
     const int th = sizeof(R) == 4 ? tile_shape32(MT).threads_solve : tile_shape(MT).threads_solve;
-    if constexpr (MT < 32) {
-        if (solve_wide<MT, R>(a)) {
-            k_solve_down_odd_wide<MT, R><<<grid, th, solve_smem_bytes(MT, a.nb, a.kc, 3, sizeof(R)), s>>>(a);
+    if constexpr (Forms<MT, R>::split) {
+        if (split_form(a.m, sizeof(R))) {
+            // two panels (r and P^H r) of MT x kc per block
+            k_solve_down_split<MT><<<grid, th, (size_t)a.nb * MT * a.kc * 2 * sizeof(z2), s>>>(a);
             return cudaGetLastError();
         }
     }
-    if constexpr (MT == 16 && sizeof(R) == 8) {
-        if (th == 128) {
-            k_solve_down_odd_16c<<<grid, th, solve_smem_bytes(MT, a.nb, a.kc, 3, sizeof(R)), s>>>(a);
-            return cudaGetLastError();
+    if constexpr (Forms<MT, R>::fma) {
+        const size_t smem = solve_smem_bytes(MT, a.nb, a.kc, 3, sizeof(R));
+        if constexpr (MT < 32) {
+            if (solve_wide<MT, R>(a)) {
+                k_solve_down_odd_wide<MT, R><<<grid, th, smem, s>>>(a);
+                return cudaGetLastError();
+            }
         }
+        if constexpr (MT == 16 && sizeof(R) == 8) {
+            if (th == 128) {
+                k_solve_down_odd_16c<<<grid, th, smem, s>>>(a);
+                return cudaGetLastError();
+            }
+        }
+        k_solve_down_odd<MT, R><<<grid, th, smem, s>>>(a);
     }
-    k_solve_down_odd<MT, R><<<grid, th, solve_smem_bytes(MT, a.nb, a.kc, 3, sizeof(R)), s>>>(a);
     return cudaGetLastError();
 }
 
@@ -392,19 +431,29 @@ template <int MT, class R>
 static cudaError_t solve_up_mt(const LevelArgsT<R> &a, cudaStream_t s) {
     const dim3 grid(odd_grid(a), (unsigned)((a.k + a.kc - 1) / a.kc));
     const int th = sizeof(R) == 4 ? tile_shape32(MT).threads_solve : tile_shape(MT).threads_solve;
-    if constexpr (MT < 32) {
-        if (solve_wide<MT, R>(a)) {
-            k_solve_up_wide<MT, R><<<grid, th, solve_smem_bytes(MT, a.nb, a.kc, 3, sizeof(R)), s>>>(a);
+    if constexpr (Forms<MT, R>::split) {
+        if (split_form(a.m, sizeof(R))) {
+            // one panel (w) of MT x kc per block
+            k_solve_up_split<MT><<<grid, th, (size_t)a.nb * MT * a.kc * sizeof(z2), s>>>(a);
             return cudaGetLastError();
         }
     }
-    if constexpr (MT == 16 && sizeof(R) == 8) {
-        if (th == 128) {
-            k_solve_up_16c<<<grid, th, solve_smem_bytes(MT, a.nb, a.kc, 3, sizeof(R)), s>>>(a);
-            return cudaGetLastError();
+    if constexpr (Forms<MT, R>::fma) {
+        const size_t smem = solve_smem_bytes(MT, a.nb, a.kc, 3, sizeof(R));
+        if constexpr (MT < 32) {
+            if (solve_wide<MT, R>(a)) {
+                k_solve_up_wide<MT, R><<<grid, th, smem, s>>>(a);
+                return cudaGetLastError();
+            }
         }
+        if constexpr (MT == 16 && sizeof(R) == 8) {
+            if (th == 128) {
+                k_solve_up_16c<<<grid, th, smem, s>>>(a);
+                return cudaGetLastError();
+            }
+        }
+        k_solve_up<MT, R><<<grid, th, smem, s>>>(a);
     }
-    k_solve_up<MT, R><<<grid, th, solve_smem_bytes(MT, a.nb, a.kc, 3, sizeof(R)), s>>>(a);
     return cudaGetLastError();
 }
 

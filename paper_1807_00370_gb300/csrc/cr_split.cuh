@@ -1,0 +1,348 @@
+// cr_split.cuh -- FP64 products of small complex blocks on the tensor cores by
+// error-free splitting, one warp per 8 x 8 complex tile.
+//
+// Why.  GB300 has 2 FP64 FMA per clock per SM, and mma.sync m16n8k16 on FP16
+// operands with FP32 accumulators does 1016 multiply-adds per clock per SM
+// (both measured), so 28 of its instructions, which form one 8 x 8 x 8 complex
+// product exactly from seven slices of each operand, take 56 clocks where the
+// FP64 pipe takes 1024.  mma.sync and not tcgen05: the blocks are 8 to 64 wide,
+// its fragments are 8 wide and live in registers, where the slices are cut.
+//
+// How (the splitting of Ozaki, Ogita, Oishi, Rump 2012).  Every column p of an
+// operand has a binary exponent E_p, that of its largest entry.  An entry v
+// becomes the integer n = trunc(|v| 2^(56 - E_p)) < 2^57: the column's largest
+// entry keeps all of its 53 bits and any other entry is off by at most 2^-56 of
+// the largest.  n is cut into seven digits, n = sum d_i 2^(8(6-i)) with
+// 0 <= d_0 <= 512 and |d_i| <= 128, which FP16 holds exactly with v's sign.  The
+// digit products with i + j <= 6 are accumulated per i + j: over 64 real terms
+// (four K-steps of the instruction) these sums are at most 2^24, so FP32 holds
+// them exactly.  The dropped digit products are below 2^-55 of the largest
+// product and have either sign.  The sums are added up in 64-bit integers and
+// rounded once.  The error is thus that of one rounding of the result plus
+// about 2^-56 max|a| max|b| sqrt(K), where a chain of FP64 FMAs rounds K times.
+//
+// Cutting is integer work and bounds these kernels (the integer pipe does 64
+// lanes per clock per SM, measured): digits of a byte need no shifts, only a
+// byte permute and a mask for two entries, which is why there are seven of
+// them and not six of ten bits.
+//
+// Columns whose largest entry lies outside 2^-923 .. 2^477 (or is not finite)
+// take FP64 FMAs instead, so overflow, infinities and NaN behave as there.
+#pragma once
+#include "cr_device.cuh"
+
+namespace crs {
+
+constexpr int kSplitDigits = 7;
+// Range of the biased exponents (and, in joint scaling, of their sums) that the
+// split takes.  The lower limits keep E - e above 58 for entries with exponent
+// field 0, so that zeros are cut off; the upper ones keep results finite.
+constexpr unsigned kSplitExpLo = 100, kSplitExpHi = 1500;
+constexpr int kSplitSumHi = 2600;
+// exponent sums below which a result may leave the normal range when it is scaled
+constexpr int kSplitSumTiny = 1100;
+
+// One FP16 digit plane of a 16 x 16 A operand and a 16 x 8 B operand.
+__device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                        uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// |v| as an ordered integer (its high word without the sign).
+__device__ __forceinline__ unsigned mag_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+
+// Exponent field of a column from the largest mag_hi of its entries: a column
+// of zeros takes that of 1.0 (its digits are zero).  Entries below 2^-1042
+// have mag_hi = 0 and count as zero.
+__device__ __forceinline__ int split_exp(unsigned mx) { return mx == 0u ? 1023 : (int)(mx >> 20); }
+__device__ __forceinline__ bool split_unsafe(unsigned mx) {
+    return mx != 0u && (mx < (kSplitExpLo << 20) || mx >= (kSplitExpHi << 20));
+}
+
+// n = trunc(|v| 2^(56 - E)) for exponent field e of the column, plus 128 in each
+// lower digit so that the digits can be read as unsigned bytes.
+__device__ __forceinline__ void split_fix(double v, int e, uint32_t &lo, uint32_t &hi) {
+    const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
+    const int d = e - (int)(mag_hi(v) >> 20);
+    uint64_t n = ((uint64_t)((__funnelshift_l(l, h, 4) & 0x00ffffffu) | 0x01000000u) << 32) | (l << 4);
+    asm("shr.u64 %0, %0, %1;" : "+l"(n) : "r"(d));   // clamps at 64: tiny entries and zeros give 0
+    n += 0x0000808080808080ull;
+    lo = (uint32_t)n;
+    hi = (uint32_t)(n >> 32);
+}
+
+// The digits of a (low halves) and b (high halves) as FP16 pairs: bytes paired
+// by one permute, read as the mantissa of 1024 + byte, and the offset taken
+// off with the entry's sign by one exact FMA.
+__device__ __forceinline__ void split_pair(double a, double b, int ea, int eb, uint32_t (&d)[kSplitDigits]) {
+    uint32_t la, ha, lb, hb;
+    split_fix(a, ea, la, ha);
+    split_fix(b, eb, lb, hb);
+    const uint32_t sg = __byte_perm((uint32_t)__double2hiint(a), (uint32_t)__double2hiint(b), 0x7430) & 0x80008000u;
+    const uint32_t one = sg ^ 0x3c003c00u, off0 = sg ^ 0xe400e400u, off = sg ^ 0xe480e480u;   // +-1, -+1024, -+1152
+    d[6] = __byte_perm(la, lb, 0x5410);
+    d[5] = __byte_perm(la, lb, 0x6521);
+    d[4] = __byte_perm(la, lb, 0x7632);
+    d[3] = __byte_perm(la, lb, 0x4703);
+    d[2] = __byte_perm(ha, hb, 0x5410);
+    d[1] = __byte_perm(ha, hb, 0x6521);
+    d[0] = __byte_perm(ha, hb, 0x7632);
+#pragma unroll
+    for (int i = 0; i < kSplitDigits; ++i) {
+        const uint32_t u = (d[i] & (i == 0 ? 0x03ff03ffu : 0x00ff00ffu)) | 0x64006400u;
+        asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d[i]) : "r"(u), "r"(one), "r"(i == 0 ? off0 : off));
+    }
+}
+
+// The three complex products of a tile, as the real A operand of row g (Re)
+// and row g + 8 (Im) over K = [re of 8 terms | im of 8 terms].
+enum SplitKind {
+    kConjA,    // sum conj(a) b
+    kPlain,    // sum a b
+    kConjB     // sum a conj(b)
+};
+
+// The digits of the two terms k = 2t, 2t + 1 that a lane holds of its row or column.
+struct SplitCut {
+    uint32_t re[kSplitDigits], im[kSplitDigits];
+};
+__device__ __forceinline__ void split_cut(SplitCut &c, z2 z0, z2 z1, int e0, int e1) {
+    split_pair(z0.x, z1.x, e0, e1, c.re);
+    split_pair(z0.y, z1.y, e0, e1, c.im);
+}
+
+using SplitAcc = float[kSplitDigits][4];
+// Accumulators of one K-step start at 1.5 * 2^23, so that their bits are their
+// integer values plus kSplitMagic (|sum| <= 2^22 over 16 terms).
+constexpr float kSplitStart = 12582912.f;
+constexpr int kSplitMagic = 0x4b400000;
+
+__device__ __forceinline__ void split_start(SplitAcc &acc, float v) {
+#pragma unroll
+    for (int d = 0; d < kSplitDigits; ++d)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[d][j] = v;
+}
+
+// acc[i + j] += A_i B_j for i + j <= 6.
+template <SplitKind KIND>
+__device__ __forceinline__ void split_mma(const SplitCut &a, const SplitCut &b, SplitAcc &acc) {
+#pragma unroll
+    for (int i = 0; i < kSplitDigits; ++i) {
+        constexpr uint32_t kNeg = 0x80008000u;
+        const uint32_t a1 = KIND == kConjA ? a.im[i] ^ kNeg : a.im[i];
+        const uint32_t a2 = KIND == kPlain ? a.im[i] ^ kNeg : a.im[i];
+        const uint32_t a3 = KIND == kConjB ? a.re[i] ^ kNeg : a.re[i];
+#pragma unroll
+        for (int j = 0; i + j < kSplitDigits; ++j) mma_f16(acc[i + j], a.re[i], a1, a2, a3, b.re[j], b.im[j]);
+    }
+}
+
+// The integer sum of a tile's digit products in units of 2^(Ea + Eb - 54) as a
+// double, from the sums per digit (kMagic: each offset by kSplitMagic): below
+// 2^63 for up to 128 real terms.
+template <bool kMagic>
+__device__ __forceinline__ double split_value(const int (&s)[kSplitDigits]) {
+    constexpr uint64_t M = kMagic ? (uint64_t)kSplitMagic : 0;
+    constexpr uint64_t off = (M << 38) + (M << 30) + (M << 22) + (M << 14) + (M << 6);
+    const int low = (int)((uint32_t)s[5] * 256u + (uint32_t)s[6] + (512u - (uint32_t)(M * 257)));
+    uint64_t v = (uint64_t)(int64_t)(low >> 10) - off;
+    v += (uint64_t)((int64_t)s[4] * (1 << 6));
+    v += (uint64_t)((int64_t)s[3] * (1 << 14));
+    v += (uint64_t)((int64_t)s[2] * (1 << 22));
+    v += (uint64_t)((int64_t)s[1] * (1 << 30));
+    v += (uint64_t)(uint32_t)(s[0] << 6) << 32;
+    return (double)(int64_t)v;
+}
+
+// v times 2^(k - 2100) for a value of split_value and a sum k of two biased
+// exponents, by the exponent field (no FP64 instruction); and that factor.
+__device__ __forceinline__ double split_scaled(double v, int k) {
+    const int hi = __double2hiint(v);
+    return (hi << 1) == 0 ? v : __hiloint2double(hi + ((k - 2100) << 20), __double2loint(v));
+}
+__device__ __forceinline__ double split_scale(int k) { return __hiloint2double((k - 1077) << 20, 0); }
+
+// One 8 x 8 tile of a product of two 8-wide complex operands over 8 ks terms,
+// by one warp: lane (g, t) = (lane / 4, lane % 4) gets the entries
+// (row g, columns 2t + j), j = 0, 1, as v[j] times 2^(e[j] - 2100).
+// la(i, k): entry k of row i of the first operand, lb(i, k): entry k of column
+// i of the second; both return zero outside the block.
+//
+// Scaling.  kJoint = false: rows of the first and columns of the second
+// operand each on their own binary grid.  kJoint = true, for products X b
+// where the second operand holds the rows of X and the contraction runs over
+// its columns: every term k has an exponent c_k, that of the tile's largest
+// |X_ik|; X goes on the grid of c_k and b_k on that of max_k(|b_k| 2^c_k).  A
+// scaling of the unknowns (X_ik -> X_ik / d_k, b_k -> d_k b_k) leaves such a
+// product's digits as they are, as it leaves the rounding errors of FP64 FMAs.
+//
+// Entries whose row or column leaves the split's range are formed by FP64 FMAs
+// (e[j] = 2100).
+//
+// same: both operands are the same columns (cut once).
+__device__ __forceinline__ unsigned split_mag(z2 z) { return max(mag_hi(z.x), mag_hi(z.y)); }
+
+// c0, c1: exponents of the lane's two terms of the joint scaling (from the tile
+// of X, whose terms b0, b1 the lane holds); m0, m1: the largest magnitudes.
+__device__ __forceinline__ void split_joint_exp(z2 b0, z2 b1, unsigned &m0, unsigned &m1) {
+    m0 = split_mag(b0);
+    m1 = split_mag(b1);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) {
+        m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+        m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+    }
+}
+
+// Running state of the joint exponent of a row: ea (with bit 20 set when out of
+// range) and the largest exponent of X's nonzero terms.
+struct SplitJoint {
+    int ea = 0, cmax = 0;
+    __device__ __forceinline__ void term(unsigned n, unsigned mx) {
+        // a term with a zero X column needs no room (its digits are zero or
+        // cut off); one that is not finite is out of range in any case
+        const int c = split_exp(mx);
+        if (mx) cmax = max(cmax, c);
+        if (n && mx) ea = max(ea, (int)(n >> 20) + c);
+        if (split_unsafe(mx) || n >= 0x7ff00000u) ea |= 1 << 20;
+    }
+    // over the four lanes of a row: its exponent sum, and whether it is out of range
+    __device__ __forceinline__ bool finish() {
+        if (ea > kSplitSumHi) ea |= 1 << 20;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            ea = max(ea, __shfl_xor_sync(0xffffffffu, ea, o));
+            cmax = max(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
+        }
+        const bool bad = (ea >> 20) != 0 || (ea != 0 && ea < cmax + 64);
+        ea &= 0xfffff;
+        if (ea == 0) ea = 2046;
+        return bad;
+    }
+};
+
+// The largest magnitude over the four lanes of a row or column.
+__device__ __forceinline__ unsigned split_max4(unsigned m) {
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    return max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+}
+
+template <SplitKind KIND, bool kJoint, int KS, class LA, class LB>
+__device__ __forceinline__ void split_tile(int ks, LA la, LB lb, bool same, z2 (&v)[2], int (&e)[2]) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    if constexpr (KS == 1) ks = 1;
+    z2 a0, a1, b0, b1;
+    int ea = 0, eb = 0;
+    unsigned m0 = 0, m1 = 0;
+    bool rbad = false, cbad = false;
+    auto load = [&](int s) {
+        a0 = la(g, 8 * s + 2 * t);
+        a1 = la(g, 8 * s + 2 * t + 1);
+        b0 = lb(g, 8 * s + 2 * t);
+        b1 = lb(g, 8 * s + 2 * t + 1);
+    };
+    if constexpr (kJoint) {
+        SplitJoint jt;
+        for (int s = 0; s < ks; ++s) {
+            load(s);
+            split_joint_exp(b0, b1, m0, m1);
+            jt.term(split_mag(a0), m0);
+            jt.term(split_mag(a1), m1);
+        }
+        rbad = jt.finish();
+        ea = jt.ea;
+    } else {
+        for (int s = 0; s < ks; ++s) {
+            load(s);
+            m0 = max(m0, max(split_mag(a0), split_mag(a1)));
+            m1 = max(m1, max(split_mag(b0), split_mag(b1)));
+        }
+        m0 = split_max4(m0);
+        m1 = split_max4(m1);
+        rbad = split_unsafe(m0);
+        cbad = split_unsafe(m1);
+        ea = split_exp(m0);
+        eb = split_exp(m1);
+    }
+    SplitCut ca, cb;
+    SplitAcc acc;
+    int sum[4][kSplitDigits];
+    split_start(acc, KS == 1 ? kSplitStart : 0.f);
+    if constexpr (KS > 4) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int d = 0; d < kSplitDigits; ++d) sum[j][d] = 0;
+    }
+#pragma unroll 1
+    for (int s = 0; s < ks; ++s) {
+        if constexpr (KS > 1) {
+            load(s);
+            if constexpr (kJoint) split_joint_exp(b0, b1, m0, m1);
+        }
+        if constexpr (kJoint) {
+            // b is cut on the grid of c_k, a on that of 2^(ea - c_k)
+            const int c0 = split_exp(m0), c1 = split_exp(m1);
+            split_cut(ca, a0, a1, ea - c0, ea - c1);
+            split_cut(cb, b0, b1, c0, c1);
+        } else {
+            split_cut(ca, a0, a1, ea, ea);
+            if (same) cb = ca;
+            else split_cut(cb, b0, b1, eb, eb);
+        }
+        split_mma<KIND>(ca, cb, acc);
+        if constexpr (KS > 4) {
+            if ((s & 3) == 3) {     // 64 terms: what FP32 holds exactly
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int d = 0; d < kSplitDigits; ++d) sum[j][d] += __float2int_rn(acc[d][j]);
+                split_start(acc, 0.f);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int d = 0; d < kSplitDigits; ++d) {
+            if constexpr (KS == 1) sum[j][d] = __float_as_int(acc[d][j]);
+            else if constexpr (KS <= 4) sum[j][d] = __float2int_rn(acc[d][j]);
+            else sum[j][d] += __float2int_rn(acc[d][j]);
+        }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        v[j] = zmk(split_value<KS == 1>(sum[j]), split_value<KS == 1>(sum[j + 2]));
+        e[j] = ea + (kJoint ? 0 : __shfl_sync(kAll, eb, 8 * t + 4 * j));
+    }
+    if (__any_sync(kAll, rbad || cbad || min(e[0], e[1]) < kSplitSumTiny)) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const bool col_bad = __shfl_sync(kAll, (int)cbad, 8 * t + 4 * j) != 0;
+            if (rbad || col_bad) {
+                // each entry decides for itself, so that it does not depend
+                // on which columns share its tile
+                z2 r = zmk(0.0, 0.0);
+                for (int k = 0; k < 8 * ks; ++k) {
+                    const z2 x = la(g, k), y = lb(2 * t + j, k);
+                    if constexpr (KIND == kConjA) zmac_ca(r, x, y);
+                    else if constexpr (KIND == kPlain) zmac(r, x, y);
+                    else zmac_cb(r, x, y);
+                }
+                v[j] = r;
+                e[j] = 2100;
+            } else if (e[j] < kSplitSumTiny) {
+                // two exact factors down to the last, which rounds into the subnormal range
+                const double s0 = split_scale(2100 - 950), s1 = split_scale(e[j] + 950);
+                v[j].x = v[j].x * s0 * s1;
+                v[j].y = v[j].y * s0 * s1;
+                e[j] = 2100;
+            }
+        }
+    }
+}
+
+}  // namespace crs
