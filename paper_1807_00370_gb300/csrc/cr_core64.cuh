@@ -40,11 +40,12 @@ template <int MT, class R> struct Forms {
 template <int MT> struct Split64 {
     static constexpr int LDZ = 2 * MT + 1;          // row of Z
     static constexpr int SL = Tri<MT>::n | 1;       // packed triangle
-    static constexpr int SC = 9;                    // one column of an 8 x 8 diagonal block
-    static constexpr int SU = MT > 8 ? 8 * MT : 0;  // one row of blocks of -X_II^{-1} X (see inverse_chunk)
+    // scratch: two columns of an 8 x 8 diagonal block (chol_inv8) or, not at
+    // the same time, one row of blocks U (inverse_chunk)
+    static constexpr int SC = MT > 8 ? 8 * MT + 1 : 17;
 };
 __host__ __device__ constexpr size_t factor64_entries(int mt) {
-    return (size_t)(((mt * (mt + 1) / 2) | 1) + mt * (2 * mt + 1) + 9 + (mt > 8 ? 8 * mt : 0));
+    return (size_t)(((mt * (mt + 1) / 2) | 1) + mt * (2 * mt + 1) + (mt > 8 ? 8 * mt + 1 : 17));
 }
 
 // Row of entry f of a packed 8 x 8 lower triangle.
@@ -53,26 +54,95 @@ __device__ __forceinline__ int tri8_row(int f) {
     return f >= 28 ? 7 : __popc(kStarts & ((2u << f) - 1u));
 }
 
+// The breakdown test of pivot d of block b, and 1 / d: the approximate reciprocal
+// and one third-order step (y (1 + e + e^2), e = 1 - d y).  Pivots in
+// 2^-999 .. 2^985 are told by their high word, as a comparison in FP64 would
+// take as long as a step of the reciprocal.
+__device__ __forceinline__ double pivot_rcp(const LevelArgs &a, int64_t block, double d) {
+    if ((unsigned)(__double2hiint(d) - 0x01800000) >= 0x7c000000u) {
+        if (!(d > 0.0)) report_fail(a.status, a.level, report_index(a, 2 * block));
+        return 1.0 / d;
+    }
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    double e = fma(-d, y, 1.0);
+    e = fma(e, e, e);
+    return fma(y, e, y);
+}
+
 // X = L^{-1} of the diagonal blocks o .. o + w - 1 (w <= 8) of A_b = L L^H (packed
 // lower in sL, in place) for the blocks b < nbh of a chunk, with the breakdown
-// test of every pivot.  Right-looking: with column c of L final, every later row
-// r takes l_r times (the conjugate of) column c of L off its trailing entries
-// and l_r times row c of X off its entries of X; column c of L is not needed
-// after that, so X takes its place (a Gauss-Jordan step).  A step is two
-// barriers: the scaling of column c and of row c of X; the updates, one entry
-// per thread, and meanwhile in a warp of its own (about as long as the other
-// warps' updates) the next pivot.  Consecutive threads take consecutive blocks.
+// test of every pivot.  Right-looking elimination A = M D M^H: with pivot d_c
+// final, every later row r takes t_r = A_rc / d_c times (the conjugate of) column
+// c off its trailing entries and t_r times row c of M^{-1} off its entries of
+// M^{-1}; column c of A is not needed after that, so -t_r, the new entry of M^{-1},
+// takes its place (a Gauss-Jordan step).  At the end X = D^{-1/2} M^{-1}: the
+// square roots are off the chain of pivots, which on GB300 costs 64 clocks per
+// FP64 instruction of a warp whatever its lanes (measured).  Two forms with the
+// same operations on every entry, so the same numbers:
+//  - up to 4 blocks (coarse levels; also what a CTA of m > 32 holds): a warp per
+//    block, two entries per lane, pivots and columns by shuffles;
+//  - else: one entry per thread, consecutive threads on consecutive blocks, two
+//    barriers per column (t and the column copied; the updates, and meanwhile
+//    in a warp of its own the next pivot), which takes a tenth of the FP64
+//    instructions.
 // Ends with __syncthreads().
 template <int MT>
 __device__ __forceinline__ void chol_inv8(const LevelArgs &a, int64_t t0, z2 *sL, z2 *sC, int nbh, int o, int w) {
     constexpr int SL = Split64<MT>::SL, SC = Split64<MT>::SC;
     const int NT = blockDim.x, tid = threadIdx.x;
-    const int npiv = NT >= 64 ? 32 : 0;       // threads kept for the pivots
     auto at = [&](int r, int c) { return tri(o + r, o + c); };
-    auto pivot = [&](int b, int c, double d) {
-        if (!(d > 0.0)) report_fail(a.status, a.level, report_index(a, 2 * (t0 + b)));
-        sL[b * SL + at(c, c)] = zmk(rsq(d), 0.0);
-    };
+    if (nbh <= 4) {
+        constexpr unsigned kAll = 0xffffffffu;
+        const int lane = tid & 31, r = lane >> 2, q = lane & 3, nw = NT >> 5;
+        for (int b = tid >> 5; b < nbh; b += nw) {
+            z2 *Lb = sL + b * SL;
+            z2 e[2];
+            double dr = 1.0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) e[h] = (r < w && 2 * q + h <= r) ? Lb[at(r, 2 * q + h)] : zmk(0.0, 0.0);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                if (c >= w) break;
+                const z2 col = e[c & 1];    // entry (r, c) in lane 4 r + c / 2
+                const double d = __shfl_sync(kAll, col.x, 4 * c + (c >> 1));
+                if (r == c) dr = d;
+                const double s = pivot_rcp(a, t0 + b, d);
+                if (c + 1 >= w) break;
+                z2 t, wv[2];
+                t.x = __shfl_sync(kAll, col.x, 4 * r + (c >> 1)) * s;
+                t.y = __shfl_sync(kAll, col.y, 4 * r + (c >> 1)) * s;
+                const z2 cc = zconj(col);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    // conj(A_jc) from row j > c, the entry of M^{-1} from row c
+                    const int j = 2 * q + h, src = j > c ? 4 * j + (c >> 1) : 4 * c + q;
+                    const z2 v = r == c ? e[h] : cc;
+                    wv[h].x = __shfl_sync(kAll, v.x, src);
+                    wv[h].y = __shfl_sync(kAll, v.y, src);
+                    if (j == c) wv[h] = zmk(1.0, 0.0);
+                }
+                if (r > c) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (2 * q + h == c) e[h] = zmk(0.0, 0.0);
+                        zmsub(e[h], t, wv[h]);
+                    }
+                }
+            }
+            const double iv = rsq(dr);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int j = 2 * q + h;
+                if (r < w && j <= r) Lb[at(r, j)] = j == r ? zmk(iv, 0.0) : zscale(e[h], iv);
+            }
+        }
+        __syncthreads();
+        return;
+    }
+    const int npiv = NT >= 64 ? 32 : 0;       // threads kept for the pivots
+    // a pivot is kept with its reciprocal
+    auto pivot = [&](int b, int c, double d) { sL[b * SL + at(c, c)] = zmk(d, pivot_rcp(a, t0 + b, d)); };
     const int pstep = npiv ? npiv : NT;
     const bool piv = tid < pstep;
     if (piv)
@@ -80,25 +150,27 @@ __device__ __forceinline__ void chol_inv8(const LevelArgs &a, int64_t t0, z2 *sL
     const int q1 = min(nbh, NT), b1 = tid % q1, f1 = tid / q1, s1 = NT / q1;
     const int nu = NT - npiv, q2 = min(nbh, nu), ut = tid - npiv, b2 = ut % q2, f2 = ut / q2, s2 = nu / q2;
     const int ntri = w * (w + 1) / 2;
-    for (int c = 0; c < w; ++c) {
+    for (int c = 0; c + 1 < w; ++c) {
         __syncthreads();
         if (f1 < s1 && f1 < w)
             for (int b = b1; b < nbh; b += q1) {
-                z2 *Lb = sL + b * SL;
-                const double iv = Lb[at(c, c)].x;
+                const z2 *Lb = sL + b * SL;
+                z2 *Cb = sC + b * SC;
+                const double s = Lb[at(c, c)].y;
                 for (int i = f1; i < w; i += s1) {
-                    if (i > c) sC[b * SC + i] = zscale(Lb[at(i, c)], iv);
-                    else if (i < c) Lb[at(c, i)] = zscale(Lb[at(c, i)], iv);
+                    if (i <= c) continue;
+                    const z2 v = Lb[at(i, c)];
+                    Cb[i] = zscale(v, s);
+                    Cb[8 + i] = v;
                 }
             }
         __syncthreads();
-        if (c + 1 == w) break;
         if (piv)
             for (int b = tid; b < nbh; b += pstep) {
-                const z2 l = sC[b * SC + c + 1];
+                const z2 t = sC[b * SC + c + 1], v = sC[b * SC + 8 + c + 1];
                 double d = sL[b * SL + at(c + 1, c + 1)].x;
-                d = fma(-l.x, l.x, d);
-                d = fma(-l.y, l.y, d);
+                d = fma(-t.x, v.x, d);
+                d = fma(-t.y, v.y, d);
                 pivot(b, c + 1, d);
             }
         if (ut >= 0 && f2 < s2)
@@ -108,15 +180,31 @@ __device__ __forceinline__ void chol_inv8(const LevelArgs &a, int64_t t0, z2 *sL
                 for (int f = tri(c + 1, 0) + f2; f < ntri; f += s2) {
                     const int r = tri8_row(f), j = f - tri(r, 0);
                     if (j == c + 1 && r == c + 1) continue;             // the next pivot
-                    const z2 l = Cb[r];
-                    z2 y = j > c ? Cb[j] : Lb[at(c, j)], u = Lb[at(r, j)];
-                    if (j > c) y = zconj(y);
-                    if (j == c) u = zmk(0.0, 0.0);
-                    zmsub(u, l, y);
+                    const z2 t = Cb[r];
+                    z2 y = j > c ? zconj(Cb[8 + j]) : Lb[at(c, j)], u = Lb[at(r, j)];
+                    if (j == c) {
+                        y = zmk(1.0, 0.0);
+                        u = zmk(0.0, 0.0);
+                    }
+                    zmsub(u, t, y);
                     Lb[at(r, j)] = u;
                 }
             }
     }
+    __syncthreads();
+    if (f1 < s1 && f1 < w)
+        for (int b = b1; b < nbh; b += q1)
+            for (int r = f1; r < w; r += s1) sC[b * SC + r].x = rsq(sL[b * SL + at(r, r)].x);
+    __syncthreads();
+    if (f1 < s1)
+        for (int b = b1; b < nbh; b += q1)
+            for (int f = f1; f < ntri; f += s1) {
+                const int r = tri8_row(f), j = f - tri(r, 0);
+                const double iv = sC[b * SC + r].x;
+                z2 *u = sL + b * SL + at(r, j);
+                *u = r == j ? zmk(iv, 0.0) : zscale(*u, iv);
+            }
+    __syncthreads();
 }
 
 // X_b = L_b^{-1} of A_b = L_b L_b^H (packed lower in sL, in place) for the blocks
@@ -126,13 +214,14 @@ __device__ __forceinline__ void chol_inv8(const LevelArgs &a, int64_t t0, z2 *sL
 // so that every block is rounded once per formula.  X_JK takes the place of
 // L_JK one step after U_JK has read row J of L.  Ends with __syncthreads().
 template <int MT, bool FULL>
-__device__ __forceinline__ void inverse_chunk(const LevelArgs &a, int64_t t0, z2 *sL, z2 *sC, z2 *sU, int nbh) {
+__device__ __forceinline__ void inverse_chunk(const LevelArgs &a, int64_t t0, z2 *sL, z2 *sC, int nbh) {
     const int m = FULL ? MT : a.m;
     if constexpr (MT == 8) {
         chol_inv8<MT>(a, t0, sL, sC, nbh, 0, m);
         return;
     } else {
-        constexpr int SL = Split64<MT>::SL, SU = Split64<MT>::SU, KS = MT / 8;
+        constexpr int SL = Split64<MT>::SL, SU = Split64<MT>::SC, KS = MT / 8;
+        z2 *sU = sC;
         const z2 zero = zmk(0.0, 0.0);
         const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, tq = lane & 3, warp = tid >> 5, nw = blockDim.x >> 5;
         const int g8 = FULL ? KS : (m + 7) >> 3;
@@ -223,7 +312,6 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
     z2 *sL = reinterpret_cast<z2 *>(smem_raw);              // [nb][SL] A_2t, then X, then P^H P
     z2 *sZ = sL + (size_t)nb * SL;                            // [nb][MT][LDZ] [B_l | B_r^H], then Z = [P | Q]
     z2 *sC = sZ + (size_t)nb * MT * LDZ;                      // [nb][SC]
-    z2 *sU = sC + (size_t)nb * Split64<MT>::SC;               // [nb][SU]
     const z2 zero = zmk(0.0, 0.0);
 
     for (int e = tid; e < nbh * mm; e += NT) {
@@ -235,7 +323,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
             (pos + 1 < a.Nl && CRS_IN(a, kDbgB, pos * mm + rem)) ? zconj(a.B[pos * mm + rem]) : zero;
     }
     __syncthreads();
-    inverse_chunk<MT, FULL>(a, t0, sL, sC, sU, nbh);
+    inverse_chunk<MT, FULL>(a, t0, sL, sC, nbh);
 
     const int lane = tid & 31, g = lane >> 2, tq = lane & 3, warp = tid >> 5, nw = NT >> 5;
     const int g8 = (FULL || KS == 1) ? KS : (m + 7) >> 3, ngrp = 2 * g8;
@@ -298,10 +386,13 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
         const int64_t o = (t0 + b - 1) * mm + p * m + q;
         if (CRS_IN(a, kDbgBn, o)) a.Bn[o] = zneg(w);
     };
-    // A - Q^H Q at entry (p, q), q <= p, of block b's right even block
-    auto sub_qq = [&](int b, int p, int q, z2 v, int ex) {
+    // A - Q^H Q at entry (p, q), q <= p, of block b's right even block (A loaded
+    // ahead of the product)
+    auto load_a = [&](int b, int p, int q) {
         const int64_t oa = (2 * (t0 + b) + 1) * mm + p * m + q;
-        z2 u = CRS_IN(a, kDbgA, oa) ? a.A[oa] : zero;
+        return (q <= p && (FULL || p < m) && 2 * (t0 + b) + 1 < a.Nl && CRS_IN(a, kDbgA, oa)) ? a.A[oa] : zero;
+    };
+    auto sub_qq = [&](z2 u, int p, int q, z2 v, int ex) {
         const double sc = -split_scale(ex);
         u.x = fma(v.x, sc, u.x);
         u.y = p == q ? 0.0 : fma(v.y, sc, u.y);
@@ -333,8 +424,10 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
         const z2 *Zb = sZ + b * MT * LDZ;
         const z2 *zi = Zb + 8 * I + (pI ? 0 : m), *zj = Zb + 8 * J + (pJ ? 0 : m);
         const int ni = m - 8 * I, nj = m - 8 * J;
-        z2 v[2];
+        z2 v[2], u[2];
         int ex[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) u[j] = pJ ? zero : load_a(b, 8 * I + g, 8 * J + 2 * tq + j);
         split_tile<kConjA, false, KS>(
             g8, [&](int i, int k) { return (FULL || (i < ni && k < m)) ? zi[k * LDZ + i] : zero; },
             [&](int i, int k) { return (FULL || (i < nj && k < m)) ? zj[k * LDZ + i] : zero; }, zi == zj, v, ex);
@@ -344,7 +437,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
             const int q = 8 * J + 2 * tq + j;
             if (!FULL && (p >= m || q >= m)) continue;
             if (!pJ) {
-                if (q <= p) put_v(b, p, q, sub_qq(b, p, q, v[j], ex[j]));
+                if (q <= p) put_v(b, p, q, sub_qq(u[j], p, q, v[j], ex[j]));
                 continue;
             }
             z2 w = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
@@ -451,7 +544,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                         const z2 v = zmk(split_value<true>(s0), split_value<true>(s1));
                         if ((!FULL && (p >= m || q >= m)) || (f != 1 && q > p)) continue;
                         if (f == 2) {
-                            Zb[p * LDZ + q] = sub_qq(b, p, q, v, ex);
+                            Zb[p * LDZ + q] = sub_qq(load_a(b, p, q), p, q, v, ex);
                         } else {
                             z2 w = zmk(split_scaled(v.x, ex), split_scaled(v.y, ex));
                             if (f == 1) {
@@ -527,9 +620,9 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
         z2 v[2];
         int ex[2];
         split_tile<kPlain, true, KS>(
-            R + 1, [&](int i, int s) { return (i < nc && (FULL || s < m) && CRS_IN(a, kDbgY, yo + s * k + i)) ? __ldg(a.y + yo + s * k + i) : zero; },
+            R + 1, [&](int i, int s) { return (i < nc && (FULL || s < m) && CRS_IN(a, kDbgY, yo + s * k + i)) ? a.y[yo + s * k + i] : zero; },
             [&](int i, int s) {
-                return ((FULL || 8 * R + i < m) && s <= 8 * R + i && CRS_IN(a, kDbgL, xo + i * m + s)) ? __ldg(a.L + xo + i * m + s) : zero;
+                return ((FULL || 8 * R + i < m) && s <= 8 * R + i && CRS_IN(a, kDbgL, xo + i * m + s)) ? a.L[xo + i * m + s] : zero;
             },
             false, v, ex);
 #pragma unroll
@@ -550,11 +643,18 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
             if (pass ? 2 * t + 1 >= a.Nl : t < 1) continue;
             const int nc = kw - n0, np = m - 8 * G;
             const z2 *Rb = sR + b * MT * kc + n0;
-            z2 v[2];
+            z2 v[2], u[2];
             int ex[2];
+            if (pass) {     // y_even, loaded ahead of the product
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int64_t oy = (2 * t + 1) * mk + (int64_t)(8 * G + g) * k + cb + n0 + 2 * tq + j;
+                    u[j] = ((FULL || g < np) && 2 * tq + j < nc && CRS_IN(a, kDbgY, oy)) ? a.y[oy] : zero;
+                }
+            }
             split_tile<kConjA, false, KS>(
                 g8,
-                [&](int i, int s) { return ((FULL || (i < np && s < m)) && CRS_IN(a, kDbgZ, zo + s * m2 + i)) ? __ldg(a.Z + zo + s * m2 + i) : zero; },
+                [&](int i, int s) { return ((FULL || (i < np && s < m)) && CRS_IN(a, kDbgZ, zo + s * m2 + i)) ? a.Z[zo + s * m2 + i] : zero; },
                 [&](int i, int s) { return (i < nc && (FULL || s < m)) ? Rb[s * kc + i] : zero; }, false, v, ex);
             const int p = 8 * G + g;
 #pragma unroll
@@ -573,13 +673,12 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
                         a.cbd[chunk * mk + rem2] = w;
                     }
                 } else {
-                    const int64_t oy = (2 * t + 1) * mk + rem2;
-                    z2 u = CRS_IN(a, kDbgY, oy) ? __ldg(a.y + oy) : zero;
+                    z2 w = u[j];
                     const double sc = -split_scale(ex[j]);
-                    u.x = fma(v[j].x, sc, u.x);
-                    u.y = fma(v[j].y, sc, u.y);
-                    if (b + 1 < nbh) u = zsub(u, sW[((b + 1) * MT + p) * kc + n0 + n]);
-                    if (CRS_IN(a, kDbgYn, t * mk + rem2)) a.yn[t * mk + rem2] = u;
+                    w.x = fma(v[j].x, sc, w.x);
+                    w.y = fma(v[j].y, sc, w.y);
+                    if (b + 1 < nbh) w = zsub(w, sW[((b + 1) * MT + p) * kc + n0 + n]);
+                    if (CRS_IN(a, kDbgYn, t * mk + rem2)) a.yn[t * mk + rem2] = w;
                 }
             }
         }
@@ -619,7 +718,7 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
         if (failed && CRS_IN(a, kDbgX, 2 * t * mk + o)) a.x[2 * t * mk + o] = zmk(qnan(0.0), qnan(0.0));
         if (t < a.ne && CRS_IN(a, kDbgX, (2 * t + 1) * mk + o))
             a.x[(2 * t + 1) * mk + o] =
-                failed ? zmk(qnan(0.0), qnan(0.0)) : (CRS_IN(a, kDbgXn, t * mk + o) ? __ldg(a.xn + t * mk + o) : zero);
+                failed ? zmk(qnan(0.0), qnan(0.0)) : (CRS_IN(a, kDbgXn, t * mk + o) ? a.xn[t * mk + o] : zero);
     }
     if (failed) return;
 
@@ -628,8 +727,13 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
         const int64_t t = t0 + b, zo = t * m2 * m + 8 * R * m2;
         const int nc = kw - n0;
         const bool hasL = t >= 1, hasR = t < a.ne;
-        z2 v[2];
+        z2 v[2], u[2];
         int ex[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {       // r, loaded ahead of the product
+            const int64_t o = t * mk + (int64_t)(8 * R + 2 * tq + j) * k + cb + n0 + g;
+            u[j] = (g < nc && (FULL || 8 * R + 2 * tq + j < m) && CRS_IN(a, kDbgR, o)) ? a.r[o] : zero;
+        }
         // terms 0 .. 8 g8 - 1: P and x_left, 8 g8 .. : Q and x_right
         split_tile<kPlain, true, 2 * KS>(
             2 * g8,
@@ -637,21 +741,20 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
                 const bool right = s >= 8 * g8;
                 const int q = right ? s - 8 * g8 : s;
                 const int64_t o = (right ? t : t - 1) * mk + q * k + cb + n0 + i;
-                return (i < nc && (FULL || q < m) && (right ? hasR : hasL) && CRS_IN(a, kDbgXn, o)) ? __ldg(a.xn + o) : zero;
+                return (i < nc && (FULL || q < m) && (right ? hasR : hasL) && CRS_IN(a, kDbgXn, o)) ? a.xn[o] : zero;
             },
             [&](int i, int s) {
                 const bool right = s >= 8 * g8;
                 const int q = right ? s - 8 * g8 : s;
                 const int64_t o = zo + i * m2 + (right ? m : 0) + q;
-                return ((FULL || (8 * R + i < m && q < m)) && CRS_IN(a, kDbgZ, o)) ? __ldg(a.Z + o) : zero;
+                return ((FULL || (8 * R + i < m && q < m)) && CRS_IN(a, kDbgZ, o)) ? a.Z[o] : zero;
             },
             false, v, ex);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int r = 8 * R + 2 * tq + j;
-            const int64_t o = t * mk + r * k + cb + n0 + g;
-            if (g >= nc || (!FULL && r >= m) || !CRS_IN(a, kDbgR, o)) continue;
-            z2 w = __ldg(a.r + o);
+            if (g >= nc || (!FULL && r >= m)) continue;
+            z2 w = u[j];
             const double sc = -split_scale(ex[j]);
             w.x = fma(v[j].x, sc, w.x);
             w.y = fma(v[j].y, sc, w.y);
@@ -668,7 +771,7 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
         int ex[2];
         // X[s][p] is zero for s < p: terms from row 8 G on
         split_tile<kConjA, false, KS>(
-            g8 - G, [&](int i, int s) { return ((FULL || (i < np && s < np)) && i <= s && CRS_IN(a, kDbgL, xo + s * m + i)) ? __ldg(a.L + xo + s * m + i) : zero; },
+            g8 - G, [&](int i, int s) { return ((FULL || (i < np && s < np)) && i <= s && CRS_IN(a, kDbgL, xo + s * m + i)) ? a.L[xo + s * m + i] : zero; },
             [&](int i, int s) { return (i < nc && (FULL || s < np)) ? Wb[s * kc + i] : zero; }, false, v, ex);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {

@@ -140,20 +140,21 @@ __device__ __forceinline__ void split_mma(const SplitCut &a, const SplitCut &b, 
     }
 }
 
-// The integer sum of a tile's digit products in units of 2^(Ea + Eb - 54) as a
-// double, from the sums per digit (kMagic: each offset by kSplitMagic): below
-// 2^63 for up to 128 real terms.
-template <bool kMagic>
+// The integer sum of a tile's digit products in units of 2^(Ea + Eb - 54 + kShift)
+// as a double, from the sums per digit (kMagic: each offset by kSplitMagic):
+// below 2^63 for up to 128 real terms, with kShift = 1 up to 256.
+template <bool kMagic, int kShift = 0>
 __device__ __forceinline__ double split_value(const int (&s)[kSplitDigits]) {
+    constexpr int H = kShift;
     constexpr uint64_t M = kMagic ? (uint64_t)kSplitMagic : 0;
-    constexpr uint64_t off = (M << 38) + (M << 30) + (M << 22) + (M << 14) + (M << 6);
-    const int low = (int)((uint32_t)s[5] * 256u + (uint32_t)s[6] + (512u - (uint32_t)(M * 257)));
-    uint64_t v = (uint64_t)(int64_t)(low >> 10) - off;
-    v += (uint64_t)((int64_t)s[4] * (1 << 6));
-    v += (uint64_t)((int64_t)s[3] * (1 << 14));
-    v += (uint64_t)((int64_t)s[2] * (1 << 22));
-    v += (uint64_t)((int64_t)s[1] * (1 << 30));
-    v += (uint64_t)(uint32_t)(s[0] << 6) << 32;
+    constexpr uint64_t off = (M << (38 - H)) + (M << (30 - H)) + (M << (22 - H)) + (M << (14 - H)) + (M << (6 - H));
+    const int low = (int)((uint32_t)s[5] * 256u + (uint32_t)s[6] + ((512u << H) - (uint32_t)(M * 257)));
+    uint64_t v = (uint64_t)(int64_t)(low >> (10 + H)) - off;
+    v += (uint64_t)((int64_t)s[4] * (1 << (6 - H)));
+    v += (uint64_t)((int64_t)s[3] * (1 << (14 - H)));
+    v += (uint64_t)((int64_t)s[2] * (1 << (22 - H)));
+    v += (uint64_t)((int64_t)s[1] * (1 << (30 - H)));
+    v += (uint64_t)(uint32_t)(s[0] << (6 - H)) << 32;
     return (double)(int64_t)v;
 }
 
@@ -315,8 +316,8 @@ __device__ __forceinline__ void split_tile(int ks, LA la, LB lb, bool same, z2 (
         }
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-        v[j] = zmk(split_value<KS == 1>(sum[j]), split_value<KS == 1>(sum[j + 2]));
-        e[j] = ea + (kJoint ? 0 : __shfl_sync(kAll, eb, 8 * t + 4 * j));
+        v[j] = zmk(split_value<KS == 1, (KS > 8)>(sum[j]), split_value<KS == 1, (KS > 8)>(sum[j + 2]));
+        e[j] = ea + (kJoint ? 0 : __shfl_sync(kAll, eb, 8 * t + 4 * j)) + (KS > 8 ? 1 : 0);
     }
     if (__any_sync(kAll, rbad || cbad || min(e[0], e[1]) < kSplitSumTiny)) {
 #pragma unroll
