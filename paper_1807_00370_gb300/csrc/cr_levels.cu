@@ -131,6 +131,65 @@ __global__ void __launch_bounds__(256) k_adjoint_outer(int64_t N, int m, int k, 
     }
 }
 
+// The same by 8 x 8 tiles on the tensor cores (cr_split.cuh), one warp per tile:
+// the terms of a tile are the 2k columns of [gy | x] against [x | gy], on
+// the joint grid of each column, so that columns of different scale keep
+// their own precision.  KS: K-steps of the class of k.  FP64 FMAs bound the
+// form above (97% of the pipe); at N = 65536, m = 16, k = 8 it took 2.63 ms and this
+// one 0.99.
+template <int KS>
+__global__ void __launch_bounds__(256) k_adjoint_outer_split(int64_t N, int m, int k, const z2 *__restrict__ x,
+                                                             const z2 *__restrict__ gy, z2 *gA, z2 *gB) {
+    const int g8 = (m + 7) >> 3, ntri = g8 * (g8 + 1) / 2, nA = gA ? ntri : 0, per = nA + (gB ? g8 * g8 : 0);
+    const int lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
+    const int64_t mk = (int64_t)m * k, mm = (int64_t)m * m, nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const z2 zero = zmk(0.0, 0.0);
+    for (int64_t e = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); e < N * per; e += nw) {
+        const int64_t j = e / per;
+        const int f = (int)(e - j * per);
+        const bool isA = f < nA;
+        if (!isA && j + 1 >= N) continue;
+        int I, J;
+        if (isA) {
+            I = tri_row(f);
+            J = f - I * (I + 1) / 2;
+        } else {
+            I = (f - nA) / g8;
+            J = f - nA - I * g8;
+        }
+        const int64_t o1 = (isA ? j : j + 1) * mk + (int64_t)(8 * I) * k, o0 = j * mk + (int64_t)(8 * J) * k;
+        const int ni = m - 8 * I, nj = m - 8 * J;
+        z2 v[2];
+        int ex[2];
+        split_tile<kConjB, true, KS>(
+            (2 * k + 7) >> 3,
+            [&](int i, int s) {
+                const bool h = s >= k;
+                return (i < ni && s < 2 * k) ? __ldg((h ? x : gy) + o1 + i * k + (h ? s - k : s)) : zero;
+            },
+            [&](int i, int s) {
+                const bool h = s >= k;
+                return (i < nj && s < 2 * k) ? __ldg((h ? gy : x) + o0 + i * k + (h ? s - k : s)) : zero;
+            },
+            false, v, ex);
+        const int p = 8 * I + g;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int q = 8 * J + 2 * tq + u;
+            if (p >= m || q >= m) continue;
+            const z2 w = zneg(zmk(split_scaled(v[u].x, ex[u]), split_scaled(v[u].y, ex[u])));
+            if (!isA) {
+                gB[j * mm + p * m + q] = w;
+            } else if (q <= p) {
+                z2 h = zscale(w, 0.5);
+                if (p == q) h.y = 0.0;
+                gA[j * mm + p * m + q] = h;
+                if (p != q) gA[j * mm + q * m + p] = zconj(h);
+            }
+        }
+    }
+}
+
 __global__ void k_nan_if_failed(z2 *x, int64_t n, const unsigned long long *status) {
     if (*status == CRS_NO_FAIL) return;
     const z2 nan2 = zmk(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
@@ -512,10 +571,29 @@ cudaError_t launch_solve_up(int mt, const LevelArgsT<float> &a, cudaStream_t s) 
     CRS_DISPATCH(solve_up_mt, float, mt, a, s)
 }
 
+// Outer products by tiles: up to 32 columns (64 complex terms: the range of the
+// tile's integer sums), and where the FMAs of a block row, (3 m^2 + m) k
+// complex ones, take longer than its tiles at 62 + 126 K-steps each (both sides
+// fitted to times at m = 5 .. 64 and k = 1 .. 32; e.g. N = 7812, m = 16: k = 1
+// 52 us by FMAs and 66 by tiles, k = 2 92 and 67, k = 8 328 and 123, k = 32 1276
+// and 379).
+static bool outer_split(int m, int k) {
+    const int g8 = (m + 7) / 8, tiles = g8 * (g8 + 1) / 2 + g8 * g8, ks = (2 * k + 7) / 8;
+    return k <= 32 && (3 * m * m + m) * k > tiles * (62 + 126 * ks);
+}
+
 cudaError_t launch_adjoint_outer(int64_t N, int m, int k, const z2 *x, const z2 *gy, z2 *gA, z2 *gB,
                                  int nsm, cudaStream_t s) {
     const int64_t items = (gA ? N * (m * (m + 1) / 2) : 0) + (gB ? (N - 1) * m * m : 0);
     if (items == 0) return cudaSuccess;
+    if (outer_split(m, k)) {
+        const int64_t g8 = (m + 7) / 8, tiles = N * ((gA ? g8 * (g8 + 1) / 2 : 0) + (gB ? g8 * g8 : 0));
+        const unsigned grid = grid_1d(tiles * 32, nsm);
+        if (k <= 4) k_adjoint_outer_split<1><<<grid, 256, 0, s>>>(N, m, k, x, gy, gA, gB);
+        else if (k <= 16) k_adjoint_outer_split<4><<<grid, 256, 0, s>>>(N, m, k, x, gy, gA, gB);
+        else k_adjoint_outer_split<8><<<grid, 256, 0, s>>>(N, m, k, x, gy, gA, gB);
+        return cudaGetLastError();
+    }
     k_adjoint_outer<<<grid_1d(items, nsm), 256, 0, s>>>(N, m, k, x, gy, gA, gB);
     return cudaGetLastError();
 }

@@ -95,3 +95,27 @@ def test_nonfinite_matrix_is_a_breakdown_where_the_oracle_says(cuda_ok, m, where
     _, io = oracle.cr_solve(A, B, y)
     assert io["status"] == 1 and info == io
     assert np.isnan(x).all()
+
+
+@pytest.mark.parametrize("m,k", [(7, 4), (8, 2), (8, 9), (9, 16), (12, 5), (16, 8), (17, 32), (33, 3), (64, 17)])
+def test_outer_products(cuda_ok, m, k):
+    """The gradients' outer products by tiles against the formula in numpy
+    from the call's own x and g_y, with columns of very different scale: each
+    gradient entry sums 2k products, so both sides are within 4k ulp of the
+    sum of the products' magnitudes."""
+    N = 21
+    A, B, y = synthetic.gen_system(N, m, k, seed=m + k)
+    s = 2.0 ** np.random.default_rng(k).integers(-30, 31, size=k)
+    dA, dB, dy, dg = to_dev(A, B, y * s, synthetic.gen_cotangent(N, m, k, seed=m) / s)
+    plan = crs.Plan(N, m, k)
+    crs.crsolve_factor(plan, dA, dB)
+    x = crs.crsolve_solve(plan, dy)
+    gy, gA, gB = (t.cpu().numpy() for t in crs.crsolve_backward(plan, x, dg))
+    x = x.cpu().numpy()
+    h = lambda t: np.conj(np.swapaxes(t, 1, 2))
+    tol = 4 * k * 2.0 ** -53
+    ref, mag = gy @ h(x), np.abs(gy) @ h(np.abs(x))
+    assert (np.abs(gA + 0.5 * (ref + h(ref))) <= tol * (mag + h(mag))).all()
+    ref = gy[1:] @ h(x[:-1]) + x[1:] @ h(gy[:-1])
+    mag = np.abs(gy[1:]) @ h(np.abs(x[:-1])) + np.abs(x[1:]) @ h(np.abs(gy[:-1]))
+    assert (np.abs(gB + ref) <= tol * mag).all()
