@@ -20,6 +20,15 @@ template <> struct Cplx<double> { using type = double2; };
 template <> struct Cplx<float> { using type = float2; };
 template <class R> using cplx_t = typename Cplx<R>::type;
 
+// Programmatic dependent launch: the level kernels of a sweep are launched so
+// that the next one may be set up while this one runs (launch_level); each
+// waits here, before its first access to memory, until the one before it has
+// finished and its stores are visible.
+__device__ __forceinline__ void level_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 #define CRS_NO_FAIL 0xFFFFFFFFFFFFFFFFull
 
 __device__ __forceinline__ double fmx(double a, double b, double c) { return fma(a, b, c); }

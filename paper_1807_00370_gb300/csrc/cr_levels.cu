@@ -10,6 +10,7 @@ namespace crs {
 
 template <int MT, class R>
 __global__ void __launch_bounds__(256) k_factor_odd(LevelArgsT<R> a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     factor_chunk<MT, R>(a, a.c_begin + blockIdx.x, smem_raw);
 }
@@ -17,28 +18,33 @@ __global__ void __launch_bounds__(256) k_factor_odd(LevelArgsT<R> a) {
 // The FP32 factor of class MT = 64 (tensor-core Schur product, L^{-1}): its
 // shared memory allows one CTA per SM, so the registers may be spent freely.
 __global__ void __launch_bounds__(256, 1) k_factor_odd_f32_64(LevelArgsT<float> a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     factor_chunk<64, float>(a, a.c_begin + blockIdx.x, smem_raw);
 }
 
 template <class R>
 __global__ void __launch_bounds__(256) k_factor_fix(LevelArgsT<R> a) {
+    level_begin();
     factor_fix_items<R>(a, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 template <int MT, class R>
 __global__ void __launch_bounds__(256) k_solve_down_odd(LevelArgsT<R> a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_down_chunk<MT, R>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
 
 template <class R>
 __global__ void __launch_bounds__(256) k_solve_down_fix(LevelArgsT<R> a) {
+    level_begin();
     solve_down_fix_items<R>(a, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 template <int MT, class R>
 __global__ void __launch_bounds__(256) k_solve_up(LevelArgsT<R> a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_up_chunk<MT, R>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
@@ -47,10 +53,12 @@ __global__ void __launch_bounds__(256) k_solve_up(LevelArgsT<R> a) {
 // capped so that five CTAs fit on an SM (16 warps otherwise): more warps to
 // cover the loads at the start of each chunk.
 __global__ void __launch_bounds__(128, 5) k_solve_down_odd_16c(LevelArgsT<double> a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_down_chunk<16, double>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
 __global__ void __launch_bounds__(128, 5) k_solve_up_16c(LevelArgsT<double> a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_up_chunk<16, double>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
@@ -61,16 +69,19 @@ __global__ void __launch_bounds__(128, 5) k_solve_up_16c(LevelArgsT<double> a) {
 // register allocation.
 template <int MT, class R>
 __global__ void __launch_bounds__(256) k_factor_odd_wide(LevelArgsT<R> a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     factor_chunk<MT, R, true>(a, a.c_begin + blockIdx.x, smem_raw);
 }
 template <int MT, class R>
 __global__ void __launch_bounds__(256) k_solve_down_odd_wide(LevelArgsT<R> a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_down_chunk<MT, R, true>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
 template <int MT, class R>
 __global__ void __launch_bounds__(256) k_solve_up_wide(LevelArgsT<R> a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_up_chunk<MT, R, true>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
@@ -78,16 +89,19 @@ __global__ void __launch_bounds__(256) k_solve_up_wide(LevelArgsT<R> a) {
 // The split forms of the FP64 levels (cr_core64.cuh).
 template <int MT>
 __global__ void __launch_bounds__(256) k_factor_split(LevelArgs a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     factor_chunk_split<MT>(a, a.c_begin + blockIdx.x, smem_raw);
 }
 template <int MT>
 __global__ void __launch_bounds__(256) k_solve_down_split(LevelArgs a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_down_chunk_split<MT>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
 template <int MT>
 __global__ void __launch_bounds__(256) k_solve_up_split(LevelArgs a) {
+    level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_up_chunk_split<MT>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
@@ -398,6 +412,27 @@ int solve_kc32(int mt, int k, int64_t no, int nsm) {
     return spread_kc(tile_shape32(mt).kc_max, k, num_ctas(no, solve_nb32(mt, no, nsm)), nsm);
 }
 
+// A level kernel's launch, set up while the kernel before it runs (see
+// level_begin): about 2 us less per launch (factor and solve at N = 1024, m = 8,
+// k = 4, 33 launches: 339 -> 272 us).  Not ahead: the FP32 kernels, which read
+// their inputs by read-only loads, and ranges of a level, which wait for copies
+// of another stream as well.
+template <class R>
+static void launch_level(void (*kernel)(LevelArgsT<R>), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                         const LevelArgsT<R> &a) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = sizeof(R) == 8 && a.c_count == 0 ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
 // CTAs of one launch of an odd-block kernel: the chunk range, else the level.
 template <class R>
 static unsigned odd_grid(const LevelArgsT<R> &a) {
@@ -438,19 +473,19 @@ static cudaError_t factor_odd_mt(const LevelArgsT<R> &a, cudaStream_t s) {
     const int th = sizeof(R) == 4 ? tile_shape32(MT).threads : tile_shape(MT).threads;
     if constexpr (Forms<MT, R>::split) {
         if (split_form(a.m, sizeof(R))) {
-            k_factor_split<MT><<<grid, th, a.nb * factor64_entries(MT) * sizeof(z2), s>>>(a);
+            launch_level(k_factor_split<MT>, grid, th, a.nb * factor64_entries(MT) * sizeof(z2), s, a);
             return cudaGetLastError();
         }
     }
     if constexpr (Forms<MT, R>::fma) {
         const size_t smem = factor_smem_bytes(MT, a.nb, sizeof(R));
         if constexpr (MT == 64 && sizeof(R) == 4) {
-            k_factor_odd_f32_64<<<grid, th, smem, s>>>(a);
+            launch_level(k_factor_odd_f32_64, grid, th, smem, s, a);
         } else if constexpr (MT < 32) {
-            if (factor_wide<MT, R>(a)) k_factor_odd_wide<MT, R><<<grid, th, smem, s>>>(a);
-            else k_factor_odd<MT, R><<<grid, th, smem, s>>>(a);
+            if (factor_wide<MT, R>(a)) launch_level(k_factor_odd_wide<MT, R>, grid, th, smem, s, a);
+            else launch_level(k_factor_odd<MT, R>, grid, th, smem, s, a);
         } else {
-            k_factor_odd<MT, R><<<grid, th, smem, s>>>(a);
+            launch_level(k_factor_odd<MT, R>, grid, th, smem, s, a);
         }
     }
     return cudaGetLastError();
@@ -463,7 +498,7 @@ static cudaError_t solve_down_odd_mt(const LevelArgsT<R> &a, cudaStream_t s) {
     if constexpr (Forms<MT, R>::split) {
         if (split_form(a.m, sizeof(R))) {
             // two panels (r and P^H r) of MT x kc per block
-            k_solve_down_split<MT><<<grid, th, (size_t)a.nb * MT * a.kc * 2 * sizeof(z2), s>>>(a);
+            launch_level(k_solve_down_split<MT>, grid, th, (size_t)a.nb * MT * a.kc * 2 * sizeof(z2), s, a);
             return cudaGetLastError();
         }
     }
@@ -471,17 +506,17 @@ static cudaError_t solve_down_odd_mt(const LevelArgsT<R> &a, cudaStream_t s) {
         const size_t smem = solve_smem_bytes(MT, a.nb, a.kc, 3, sizeof(R));
         if constexpr (MT < 32) {
             if (solve_wide<MT, R>(a)) {
-                k_solve_down_odd_wide<MT, R><<<grid, th, smem, s>>>(a);
+                launch_level(k_solve_down_odd_wide<MT, R>, grid, th, smem, s, a);
                 return cudaGetLastError();
             }
         }
         if constexpr (MT == 16 && sizeof(R) == 8) {
             if (th == 128) {
-                k_solve_down_odd_16c<<<grid, th, smem, s>>>(a);
+                launch_level(k_solve_down_odd_16c, grid, th, smem, s, a);
                 return cudaGetLastError();
             }
         }
-        k_solve_down_odd<MT, R><<<grid, th, smem, s>>>(a);
+        launch_level(k_solve_down_odd<MT, R>, grid, th, smem, s, a);
     }
     return cudaGetLastError();
 }
@@ -493,7 +528,7 @@ static cudaError_t solve_up_mt(const LevelArgsT<R> &a, cudaStream_t s) {
     if constexpr (Forms<MT, R>::split) {
         if (split_form(a.m, sizeof(R))) {
             // one panel (w) of MT x kc per block
-            k_solve_up_split<MT><<<grid, th, (size_t)a.nb * MT * a.kc * sizeof(z2), s>>>(a);
+            launch_level(k_solve_up_split<MT>, grid, th, (size_t)a.nb * MT * a.kc * sizeof(z2), s, a);
             return cudaGetLastError();
         }
     }
@@ -501,17 +536,17 @@ static cudaError_t solve_up_mt(const LevelArgsT<R> &a, cudaStream_t s) {
         const size_t smem = solve_smem_bytes(MT, a.nb, a.kc, 3, sizeof(R));
         if constexpr (MT < 32) {
             if (solve_wide<MT, R>(a)) {
-                k_solve_up_wide<MT, R><<<grid, th, smem, s>>>(a);
+                launch_level(k_solve_up_wide<MT, R>, grid, th, smem, s, a);
                 return cudaGetLastError();
             }
         }
         if constexpr (MT == 16 && sizeof(R) == 8) {
             if (th == 128) {
-                k_solve_up_16c<<<grid, th, smem, s>>>(a);
+                launch_level(k_solve_up_16c, grid, th, smem, s, a);
                 return cudaGetLastError();
             }
         }
-        k_solve_up<MT, R><<<grid, th, smem, s>>>(a);
+        launch_level(k_solve_up<MT, R>, grid, th, smem, s, a);
     }
     return cudaGetLastError();
 }
@@ -530,7 +565,7 @@ template <class R>
 static cudaError_t factor_fix_r(const LevelArgsT<R> &a, int nsm, cudaStream_t s) {
     const int64_t nbd = a.c_count > 0 ? a.c_count : num_ctas(a.no, a.nb) - 1;
     if (nbd < 1) return cudaSuccess;
-    k_factor_fix<R><<<grid_1d(nbd * (a.m * (a.m + 1) / 2), nsm), 256, 0, s>>>(a);
+    launch_level(k_factor_fix<R>, grid_1d(nbd * (a.m * (a.m + 1) / 2), nsm), 256, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -538,7 +573,7 @@ template <class R>
 static cudaError_t solve_down_fix_r(const LevelArgsT<R> &a, int nsm, cudaStream_t s) {
     const int64_t ncta = num_ctas(a.no, a.nb);
     if (ncta < 2) return cudaSuccess;
-    k_solve_down_fix<R><<<grid_1d((ncta - 1) * a.m * a.k, nsm), 256, 0, s>>>(a);
+    launch_level(k_solve_down_fix<R>, grid_1d((ncta - 1) * a.m * a.k, nsm), 256, 0, s, a);
     return cudaGetLastError();
 }
 
