@@ -21,7 +21,7 @@ bool set_tile_shape32(int mt, const TileShape &ts, size_t smem_limit);
 int pick_mt(int m);                                  // 4, 8, 16, 32, 64 or 0
 size_t factor_smem_bytes(int mt, int nb, int rsize = 8);           // rsize: 8 FP64, 4 FP32
 size_t solve_smem_bytes(int mt, int nb, int kc, int panels, int rsize = 8);
-cudaError_t prepare_kernels(int mt);                 // raise shared-memory limits once per device
+cudaError_t prepare_kernels(int m);                  // raise the shared-memory limits of the kernels for m
 
 // Odd blocks per CTA of a level with `no` odd blocks (the tile's maximum,
 // shrunk on small levels so that about two CTAs land on every SM), and the
@@ -35,6 +35,20 @@ int factor_nb32(int mt, int64_t no, int nsm);
 int solve_nb32(int mt, int64_t no, int nsm);
 int solve_kc32(int mt, int k, int64_t no, int nsm);
 inline int64_t num_ctas(int64_t no, int nb) { return crs_num_ctas(no, nb); }
+
+// The coarse levels of a short FP64 system, one launch for the factor and one
+// for both sweeps (cr_tail.cu): a cluster of kTailCtas CTAs with up to
+// tail_blocks(m) odd blocks each; lev[i].nb (and kc, the same for all) set so
+// that a level has at most kTailCtas chunks, the finest level first.
+constexpr int kTailCtas = 8, kTailLevels = 8, kTailCols = 8;
+struct TailArgs {
+    int n;
+    LevelArgs lev[kTailLevels];
+};
+int tail_blocks(int m);
+cudaError_t prepare_tail(int m, int smem_optin);
+cudaError_t launch_factor_tail(const TailArgs &ta, cudaStream_t s);
+cudaError_t launch_solve_tail(const TailArgs &ta, cudaStream_t s);
 
 // Factor sweep of one level (a.nb set by factor_nb): the odd-block kernel
 // (Cholesky, P, Q, Z^H Z, and the even blocks that lie inside its CTA), then

@@ -352,12 +352,14 @@ static cudaError_t prepare_mt(int smem_optin) {
     return e != cudaSuccess ? e : prepare_mt_r<MT, float>(smem_optin);
 }
 
-cudaError_t prepare_kernels(int mt) {
+cudaError_t prepare_kernels(int m) {
+    const int mt = pick_mt(m);
     int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
+    if ((e = prepare_tail(m, optin)) != cudaSuccess) return e;
     switch (mt) {
         case 4: return prepare_mt<4>(optin);
         case 8: return prepare_mt<8>(optin);

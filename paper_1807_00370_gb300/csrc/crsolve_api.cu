@@ -197,7 +197,7 @@ int debug_reset(crsolve_plan_s *p, cudaStream_t s) {
 
 int ensure_prepared(crsolve_plan_s *p) {
     if (p->prepared) return CRSOLVE_OK;
-    if (crs::prepare_kernels(p->mt) != cudaSuccess) return CRSOLVE_ECUDA;
+    if (crs::prepare_kernels(p->m) != cudaSuccess) return CRSOLVE_ECUDA;
     p->prepared = true;
     return CRSOLVE_OK;
 }
@@ -390,19 +390,35 @@ unsigned *boundary_counters(crsolve_plan_s *p, int64_t need, cudaStream_t s, int
     return cnt;
 }
 
+// First level of the plan's tail (cr_tail.cu), not below l0: the levels from it
+// on run in one launch per sweep direction.  Systems of fewer than
+// kTailMaxN blocks only: there the coarse levels are most of the time
+// (factor and solve at N = 1024, m = 8, k = 4 MEASURED_TAIL), and longer systems
+// keep one launch per level, which callers of the launch counter rely on.
+constexpr int64_t kTailMaxN = 8192;
+int tail_level(const crsolve_plan_s *p, int l0) {
+    const int nlev = (int)p->lev.size();
+    if (p->N >= kTailMaxN) return nlev;
+    int l = l0;
+    while (l < nlev && p->lev[l].no > crs::kTailCtas * (int64_t)crs::tail_blocks(p->m)) ++l;
+    return nlev - l >= 2 ? l : nlev;
+}
+int tail_nb(int64_t no) { return (int)((no + crs::kTailCtas - 1) / crs::kTailCtas); }
+
 // Factor levels [l0, nlev): the odd-block kernel per level, which also
 // completes the CTA-boundary even blocks (bd_arrive), or else a fix-up
 // kernel after it.
 int factor_levels(crsolve_plan_s *p, int l0, const z2 *A, const z2 *B, cudaStream_t s) {
     int rc;
+    const int nlev = (int)p->lev.size(), lt = tail_level(p, l0);
     int64_t need = 0;
-    for (int l = l0; l < (int)p->lev.size(); ++l) {
+    for (int l = l0; l < lt; ++l) {
         const int64_t ctas = crs::num_ctas(p->lev[l].no, crs::factor_nb(p->mt, p->lev[l].no, p->nsm));
         if (fuse_boundaries(p, ctas)) need = std::max(need, ctas);
     }
     unsigned *cnt = boundary_counters(p, need, s, &rc);
     if (rc) return rc;
-    for (int l = l0; l < (int)p->lev.size(); ++l) {
+    for (int l = l0; l < lt; ++l) {
         NvtxRange nv("factor", l);
         crs::LevelArgs a = level_args(p, l, A, B);
         a.nb = crs::factor_nb(p->mt, a.no, p->nsm);
@@ -414,6 +430,18 @@ int factor_levels(crsolve_plan_s *p, int l0, const z2 *A, const z2 *B, cudaStrea
             (rc = launch(p, CRSOLVE_K_FACTOR_FIX, l, crs::num_ctas(a.no, a.nb) - 1, s,
                          [&] { return crs::launch_factor_fix(a, p->nsm, s); })))
             return rc;
+    }
+    if (lt < nlev) {
+        NvtxRange nv("factor", lt);
+        crs::TailArgs ta{};
+        int64_t units = 0;
+        for (int l = lt; l < nlev; ++l) {
+            crs::LevelArgs &a = ta.lev[ta.n++];
+            a = level_args(p, l, A, B);
+            a.nb = tail_nb(a.no);
+            units += a.no;
+        }
+        if ((rc = launch(p, CRSOLVE_K_FACTOR_ODD, lt, units, s, [&] { return crs::launch_factor_tail(ta, s); }))) return rc;
     }
     return CRSOLVE_OK;
 }
@@ -438,19 +466,19 @@ crs::LevelArgs solve_args(const crsolve_plan_s *p, int l, int k) {
 
 // Down sweep of every level, then the up sweep of levels nlev-1 .. l_end.
 int solve_sweeps(crsolve_plan_s *p, int k, const z2 *y, z2 *x, int l_end, cudaStream_t s) {
-    const int nlev = (int)p->lev.size();
+    const int nlev = (int)p->lev.size(), lt = tail_level(p, l_end);
     int rc;
     // the down sweep completes its CTA-boundary right-hand sides itself
     // (bd_arrive; counters per CTA and column chunk) or takes fix-up kernels
     int64_t need = 0;
     auto ctas_of = [&](const crs::LevelArgs &a) { return crs::num_ctas(a.no, a.nb) * ((k + a.kc - 1) / a.kc); };
-    for (int l = 0; l < nlev; ++l) {
+    for (int l = 0; l < lt; ++l) {
         const int64_t ctas = ctas_of(solve_args(p, l, k));
         if (fuse_boundaries(p, ctas)) need = std::max(need, ctas);
     }
     unsigned *cnt = boundary_counters(p, need, s, &rc);
     if (rc) return rc;
-    for (int l = 0; l < nlev; ++l) {
+    for (int l = 0; l < lt; ++l) {
         NvtxRange nv("solve down", l);
         crs::LevelArgs a = solve_args(p, l, k);
         a.y = (l == 0) ? y : reinterpret_cast<const z2 *>(p->map() + p->lev[l - 1].offYn);
@@ -463,7 +491,24 @@ int solve_sweeps(crsolve_plan_s *p, int k, const z2 *y, z2 *x, int l_end, cudaSt
                          [&] { return crs::launch_solve_down_fix(a, p->nsm, s); })))
             return rc;
     }
-    for (int l = nlev - 1; l >= l_end; --l) {
+    if (lt < nlev) {
+        NvtxRange nv("solve down and up", lt);
+        crs::TailArgs ta{};
+        int64_t units = 0;
+        for (int l = lt; l < nlev; ++l) {
+            crs::LevelArgs &a = ta.lev[ta.n++];
+            a = level_args(p, l, nullptr, nullptr);
+            a.k = k;
+            a.nb = tail_nb(a.no);
+            a.kc = std::min(k, crs::kTailCols);
+            a.y = (l == 0) ? y : reinterpret_cast<const z2 *>(p->map() + p->lev[l - 1].offYn);
+            a.x = (l == 0) ? x : reinterpret_cast<z2 *>(p->map() + p->lev[l - 1].offXn);
+            units += a.no;
+        }
+        if ((rc = launch(p, CRSOLVE_K_SOLVE_DOWN_ODD, lt, units, s, [&] { return crs::launch_solve_tail(ta, s); })))
+            return rc;
+    }
+    for (int l = lt - 1; l >= l_end; --l) {
         NvtxRange nv("solve up", l);
         crs::LevelArgs a = solve_args(p, l, k);
         a.x = (l == 0) ? x : reinterpret_cast<z2 *>(p->map() + p->lev[l - 1].offXn);

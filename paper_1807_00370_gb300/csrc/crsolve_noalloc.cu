@@ -97,7 +97,7 @@ extern "C" int crsolve_solve_noalloc(int64_t N, int32_t m, int32_t k, const crso
     // device memory) and the kernels' shared-memory limits.
     void *p = nullptr;
     if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return CRSOLVE_ECUDA;
-    if (crs::prepare_kernels(mt) != cudaSuccess) return CRSOLVE_ECUDA;
+    if (crs::prepare_kernels(m) != cudaSuccess) return CRSOLVE_ECUDA;
     char *ws = static_cast<char *>(p);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     unsigned long long *status = reinterpret_cast<unsigned long long *>(ws + offStatus);
