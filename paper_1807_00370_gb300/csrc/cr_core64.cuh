@@ -305,6 +305,7 @@ __device__ __forceinline__ void inverse_chunk(const LevelArgs &a, int64_t t0, z2
 template <int MT, bool FULL>
 __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, unsigned char *smem_raw) {
     constexpr int LDZ = Split64<MT>::LDZ, SL = Split64<MT>::SL, KS = MT / 8;
+    constexpr bool kOn = MT >= 32;
     const int m = FULL ? MT : a.m, nb = a.nb, NT = blockDim.x, tid = threadIdx.x;
     const int mm = m * m, m2 = 2 * m;
     const int64_t t0 = chunk * nb;
@@ -328,6 +329,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
     const int lane = tid & 31, g = lane >> 2, tq = lane & 3, warp = tid >> 5, nw = NT >> 5;
     const int g8 = (FULL || KS == 1) ? KS : (m + 7) >> 3, ngrp = 2 * g8;
     z2 *sW = sL;    // P^H P
+    const z2 zero_on = split_zero_on();
 
     // Z = X [B_l | B_r^H] of 8 columns of a block in place, by one warp, the rows
     // from the bottom up.  Column groups 0 .. g8-1 are P, the others Q.
@@ -343,7 +345,13 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                 int ex[2];
                 split_tile<kPlain, true, KS>(
                     R + 1, [&](int i, int k) { return (FULL || (i < nc && k < m)) ? Zb[k * LDZ + col - g + i] : zero; },
-                    [&](int i, int k) { return ((FULL || 8 * R + i < m) && k <= 8 * R + i) ? Xb[tri(8 * R + i, k)] : zero; }, false, v, ex);
+                    [&](int i, int k) {
+                        if (!((FULL || 8 * R + i < m) && k <= 8 * R + i)) return zero;
+                        if constexpr (!kOn) return Xb[tri(8 * R + i, k)];
+                        const int64_t o = t * mm + (8 * R + i) * m + k;     // (sL has X on its grid)
+                        return CRS_IN(a, kDbgL, o) ? a.L[o] : zero;
+                    },
+                    false, v, ex);
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
@@ -409,6 +417,15 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
     // Z^H Z by tiles (row group I >= column group J): pass 0 has P^H P and Q^H P,
     // pass 1 Q^H Q.
     const int ntri = g8 * (g8 + 1) / 2;
+    //
+    // kOn: the entries of X, B and Z are put on their grids once (see the end), with
+    // the exponents of the block's columns in sE: those of X at 0, its rows at
+    // MT, Z's at 2 MT (0: out of the split's range; the tile then takes Z as
+    // stored).  Pays from m > 16 on, where a tile's operands are read by many
+    // tiles (level 0 of N = 4096, m = 64: 3335 -> 2884 us, m = 32: 448 -> 417;
+    // N = 65536, m = 16: 1069 -> 1125).
+    int *const sE = reinterpret_cast<int *>(sC);
+    constexpr int SE = 4 * Split64<MT>::SC;    // ints per block
     auto h_task = [&](int b, int pass, int f) {
         const int64_t t = t0 + b;
         int I, J;
@@ -428,9 +445,31 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
         int ex[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) u[j] = pJ ? zero : load_a(b, 8 * I + g, 8 * J + 2 * tq + j);
-        split_tile<kConjA, false, KS>(
-            g8, [&](int i, int k) { return (FULL || (i < ni && k < m)) ? zi[k * LDZ + i] : zero; },
-            [&](int i, int k) { return (FULL || (i < nj && k < m)) ? zj[k * LDZ + i] : zero; }, zi == zj, v, ex);
+        if constexpr (!kOn) {
+            split_tile<kConjA, false, KS>(
+                g8, [&](int i, int k) { return (FULL || (i < ni && k < m)) ? zi[k * LDZ + i] : zero; },
+                [&](int i, int k) { return (FULL || (i < nj && k < m)) ? zj[k * LDZ + i] : zero; }, zi == zj, v, ex);
+        } else {
+            const int *ze = sE + b * SE + 2 * MT;
+            const int ci = 8 * I + (pI ? 0 : m), cj = 8 * J + (pJ ? 0 : m);
+            const int ei = (FULL || g < ni) ? ze[ci + g] : 1023, ej = (FULL || g < nj) ? ze[cj + g] : 1023;
+            if (__any_sync(0xffffffffu, ei < 600 || ej < 600)) {
+                const int64_t oz = t * m2 * m;
+                auto zg = [&](int c, int k) {
+                    const int64_t o = oz + k * m2 + c;
+                    return CRS_IN(a, kDbgZ, o) ? a.Z[o] : zero;
+                };
+                split_tile<kConjA, false, KS>(
+                    g8, [&](int i, int k) { return (FULL || (i < ni && k < m)) ? zg(ci + i, k) : zero; },
+                    [&](int i, int k) { return (FULL || (i < nj && k < m)) ? zg(cj + i, k) : zero; }, zi == zj, v, ex);
+            } else {
+                split_tile_on<kConjA, KS>(
+                    g8, [&](int i, int k) { return (FULL || (i < ni && k < m)) ? zi[k * LDZ + i] : zero_on; },
+                    [&](int i, int k) { return (FULL || (i < nj && k < m)) ? zj[k * LDZ + i] : zero_on; }, zi == zj, v);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) ex[j] = ei + __shfl_sync(0xffffffffu, ej, 8 * tq + 4 * j);
+            }
+        }
         const int p = 8 * I + g;
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -573,7 +612,119 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
             __syncthreads();
         }
     }
-    if (MT > 8 || 2 * nbh <= nw) {
+    if constexpr (kOn) {
+        // X is stored, and put on its grid in place where all of its columns are
+        // in the split's range: column exponents, row exponents, entries.
+        constexpr unsigned kAll = 0xffffffffu;
+        for (int e = warp; e < nbh * m; e += nw) {
+            const int b = e / m, k = e - b * m;
+            unsigned mx = 0;
+            for (int r = k + lane; r < m; r += 32) mx = max(mx, split_mag(sL[b * SL + tri(r, k)]));
+            for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(kAll, mx, o));
+            if (lane == 0) sE[b * SE + k] = split_unsafe(mx) ? 0 : split_exp(mx);
+        }
+        __syncthreads();
+        for (int e = warp; e < nbh * m; e += nw) {
+            const int b = e / m, r = e - b * m;
+            int rho = -4096;
+            for (int k = lane; k <= r; k += 32) {
+                const unsigned n = split_mag(sL[b * SL + tri(r, k)]);
+                if (n) rho = max(rho, (int)(n >> 20) - sE[b * SE + k]);
+            }
+            for (int o = 16; o; o >>= 1) rho = max(rho, __shfl_xor_sync(kAll, rho, o));
+            if (lane == 0) sE[b * SE + MT + r] = max(rho, -40);     // keeps E - e above 58 for zeros
+        }
+        __syncthreads();
+        for (int e = tid; e < nbh * mm; e += NT) {
+            const int b = e / mm, rem = e - b * mm, r = rem / m, c = rem - r * m;
+            z2 x = zero;
+            if (r >= c) {
+                z2 *p = sL + b * SL + tri(r, c);
+                x = *p;
+                *p = split_onto(x, sE[b * SE + c] + sE[b * SE + MT + r]);
+            }
+            if (CRS_IN(a, kDbgL, (t0 + b) * mm + rem)) a.L[(t0 + b) * mm + rem] = x;
+        }
+        __syncthreads();
+        for (int e = warp; e < nbh * ngrp; e += nw) {
+            const int b = e / ngrp, cg = e - b * ngrp;
+            const int64_t t = t0 + b;
+            const bool inP = cg < g8;
+            const int c0 = 8 * (inP ? cg : cg - g8), nc = m - c0, col = (inP ? c0 : m + c0) + g;
+            const int *xe = sE + b * SE;
+            int *ze = sE + b * SE + 2 * MT;
+            z2 *Zb = sZ + b * MT * LDZ;
+            const z2 *Xb = sL + b * SL;
+            auto zc = [&](int k) { return (FULL || (g < nc && k < m)) ? Zb[k * LDZ + col] : zero; };
+            // B's columns onto the joint grid
+            SplitJoint jt;
+            bool xbad = false;
+            for (int s = 0; s < g8; ++s)
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int k = 8 * s + 2 * tq + u, c = (FULL || k < m) ? xe[k] : 1023;
+                    xbad |= c == 0;
+                    // (a column of X has its diagonal entry)
+                    jt.term(split_mag(zc(k)), (unsigned)c << 20);
+                }
+            bool ok = !jt.finish() && !xbad && jt.ea - 40 >= kSplitSumTiny;
+            ok = __all_sync(kAll, ok);
+            if (!(inP ? t >= 1 : 2 * t + 1 < a.Nl)) {
+                ok = false;     // no coupling: Z is zero, as staged
+            } else if (!ok) {
+                z_task(b, cg);
+            } else {
+                for (int s = 0; s < g8; ++s)
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int k = 8 * s + 2 * tq + u;
+                        if (FULL || (g < nc && k < m)) Zb[k * LDZ + col] = split_onto(Zb[k * LDZ + col], jt.ea - xe[k]);
+                    }
+                __syncwarp();
+                for (int R = g8 - 1; R >= 0; --R) {
+                    z2 v[2];
+                    split_tile_on<kPlain, KS>(
+                        R + 1, [&](int i, int k) { return (FULL || (i < nc && k < m)) ? Zb[k * LDZ + col - g + i] : zero_on; },
+                        [&](int i, int k) { return ((FULL || 8 * R + i < m) && k <= 8 * R + i) ? Xb[tri(8 * R + i, k)] : zero_on; }, false, v);
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const int r = 8 * R + 2 * tq + j;
+                        if (FULL || (g < nc && r < m)) {
+                            const int ex = jt.ea + xe[MT + r];
+                            const int64_t o = t * m2 * m + r * m2 + col;
+                            const z2 w = zmk(split_scaled(v[j].x, ex), split_scaled(v[j].y, ex));
+                            Zb[r * LDZ + col] = w;
+                            if (CRS_IN(a, kDbgZ, o)) a.Z[o] = w;
+                        }
+                    }
+                    __syncwarp();
+                }
+            }
+            if (!ok && (FULL || g < nc))
+                for (int r = tq; r < m; r += 4) {
+                    const int64_t o = t * m2 * m + r * m2 + col;
+                    if (CRS_IN(a, kDbgZ, o)) a.Z[o] = Zb[r * LDZ + col];
+                }
+            // Z's columns onto their own grid
+            unsigned mx = 0;
+            for (int s = 0; s < g8; ++s)
+#pragma unroll
+                for (int u = 0; u < 2; ++u) mx = max(mx, split_mag(zc(8 * s + 2 * tq + u)));
+            mx = split_max4(mx);
+            const int ez = split_unsafe(mx) ? 0 : split_exp(mx);
+            if (FULL || g < nc) {
+                if (tq == 0) ze[col] = ez;
+                for (int s = 0; s < g8; ++s)
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int k = 8 * s + 2 * tq + u;
+                        if (FULL || k < m) Zb[k * LDZ + col] = split_onto(Zb[k * LDZ + col], ez);
+                    }
+            }
+        }
+        __syncthreads();
+    } else if (MT > 8 || 2 * nbh <= nw) {
         for (int e = warp; e < nbh * ngrp; e += nw) z_task(e / ngrp, e % ngrp);
         // keep X
         for (int e = tid; e < nbh * mm; e += NT) {
@@ -581,6 +732,8 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
             if (CRS_IN(a, kDbgL, (t0 + b) * mm + rem)) a.L[(t0 + b) * mm + rem] = r >= c ? sL[b * SL + tri(r, c)] : zero;
         }
         __syncthreads();
+    }
+    if (MT > 8 || 2 * nbh <= nw) {
         for (int pass = 0; pass < 2; ++pass) {
             const int nt = pass == 0 ? ntri + g8 * g8 : ntri;
             for (int e = warp; e < nbh * nt; e += nw) h_task(e / nt, pass, e % nt);

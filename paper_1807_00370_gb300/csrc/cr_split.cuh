@@ -75,12 +75,10 @@ __device__ __forceinline__ void split_fix(double v, int e, uint32_t &lo, uint32_
 
 // The digits of a (low halves) and b (high halves) as FP16 pairs: bytes paired
 // by one permute, read as the mantissa of 1024 + byte, and the offset taken
-// off with the entry's sign by one exact FMA.
-__device__ __forceinline__ void split_pair(double a, double b, int ea, int eb, uint32_t (&d)[kSplitDigits]) {
-    uint32_t la, ha, lb, hb;
-    split_fix(a, ea, la, ha);
-    split_fix(b, eb, lb, hb);
-    const uint32_t sg = __byte_perm((uint32_t)__double2hiint(a), (uint32_t)__double2hiint(b), 0x7430) & 0x80008000u;
+// off with the entry's sign (bit 31 of sa, sb) by one exact FMA.
+__device__ __forceinline__ void split_digits(uint32_t la, uint32_t ha, uint32_t lb, uint32_t hb, uint32_t sa, uint32_t sb,
+                                             uint32_t (&d)[kSplitDigits]) {
+    const uint32_t sg = __byte_perm(sa, sb, 0x7430) & 0x80008000u;
     const uint32_t one = sg ^ 0x3c003c00u, off0 = sg ^ 0xe400e400u, off = sg ^ 0xe480e480u;   // +-1, -+1024, -+1152
     d[6] = __byte_perm(la, lb, 0x5410);
     d[5] = __byte_perm(la, lb, 0x6521);
@@ -94,6 +92,33 @@ __device__ __forceinline__ void split_pair(double a, double b, int ea, int eb, u
         const uint32_t u = (d[i] & (i == 0 ? 0x03ff03ffu : 0x00ff00ffu)) | 0x64006400u;
         asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d[i]) : "r"(u), "r"(one), "r"(i == 0 ? off0 : off));
     }
+}
+
+__device__ __forceinline__ void split_pair(double a, double b, int ea, int eb, uint32_t (&d)[kSplitDigits]) {
+    uint32_t la, ha, lb, hb;
+    split_fix(a, ea, la, ha);
+    split_fix(b, eb, lb, hb);
+    split_digits(la, ha, lb, hb, (uint32_t)__double2hiint(a), (uint32_t)__double2hiint(b), d);
+}
+
+// An entry on its grid, kept in the place of the double: n with its digit
+// offsets and the sign in bit 63.  Operands that many tiles read are put on
+// their grid once, which leaves the tiles the digits alone (a third of the
+// integer work of a cut).
+__device__ __forceinline__ double split_onto(double v, int e) {
+    uint32_t lo, hi;
+    split_fix(v, e, lo, hi);
+    return __hiloint2double((int)(hi | ((uint32_t)__double2hiint(v) & 0x80000000u)), (int)lo);
+}
+__device__ __forceinline__ z2 split_onto(z2 z, int e) { return zmk(split_onto(z.x, e), split_onto(z.y, e)); }
+// ... of zero: the digits' offsets.
+__device__ __forceinline__ z2 split_zero_on() {
+    const double z = __hiloint2double(0x00008080, (int)0x80808080u);
+    return zmk(z, z);
+}
+__device__ __forceinline__ void split_pair_on(double a, double b, uint32_t (&d)[kSplitDigits]) {
+    const uint32_t ha = (uint32_t)__double2hiint(a), hb = (uint32_t)__double2hiint(b);
+    split_digits((uint32_t)__double2loint(a), ha, (uint32_t)__double2loint(b), hb, ha, hb, d);
 }
 
 // The three complex products of a tile, as the real A operand of row g (Re)
@@ -111,6 +136,11 @@ struct SplitCut {
 __device__ __forceinline__ void split_cut(SplitCut &c, z2 z0, z2 z1, int e0, int e1) {
     split_pair(z0.x, z1.x, e0, e1, c.re);
     split_pair(z0.y, z1.y, e0, e1, c.im);
+}
+
+__device__ __forceinline__ void split_cut_on(SplitCut &c, z2 z0, z2 z1) {
+    split_pair_on(z0.x, z1.x, c.re);
+    split_pair_on(z0.y, z1.y, c.im);
 }
 
 using SplitAcc = float[kSplitDigits][4];
@@ -234,40 +264,62 @@ __device__ __forceinline__ unsigned split_max4(unsigned m) {
 template <SplitKind KIND, bool kJoint, int KS, class LA, class LB>
 __device__ __forceinline__ void split_tile(int ks, LA la, LB lb, bool same, z2 (&v)[2], int (&e)[2]) {
     constexpr unsigned kAll = 0xffffffffu;
+    // up to two K-steps the lane keeps its operands in registers between the
+    // pass for the exponents and the products; beyond, it loads them again
+    constexpr bool kKeep = KS <= 2;
+    constexpr int NK = kKeep ? KS : 1;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     if constexpr (KS == 1) ks = 1;
-    z2 a0, a1, b0, b1;
+    z2 a[NK][2], b[NK][2];
     int ea = 0, eb = 0;
-    unsigned m0 = 0, m1 = 0;
+    unsigned m0[NK] = {}, m1[NK] = {};
     bool rbad = false, cbad = false;
-    auto load = [&](int s) {
-        a0 = la(g, 8 * s + 2 * t);
-        a1 = la(g, 8 * s + 2 * t + 1);
-        b0 = lb(g, 8 * s + 2 * t);
-        b1 = lb(g, 8 * s + 2 * t + 1);
-    };
-    if constexpr (kJoint) {
-        SplitJoint jt;
-        for (int s = 0; s < ks; ++s) {
-            load(s);
-            split_joint_exp(b0, b1, m0, m1);
-            jt.term(split_mag(a0), m0);
-            jt.term(split_mag(a1), m1);
+    auto load = [&](int s, int i) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            a[i][u] = la(g, 8 * s + 2 * t + u);
+            b[i][u] = lb(g, 8 * s + 2 * t + u);
         }
+    };
+    if constexpr (kKeep) {
+#pragma unroll
+        for (int s = 0; s < KS; ++s) {
+            a[s][0] = a[s][1] = b[s][0] = b[s][1] = zmk(0.0, 0.0);
+            if (s < ks) load(s, s);     // (the operands end with K-step ks - 1)
+        }
+    }
+    SplitJoint jt;
+    unsigned ma = 0, mb = 0;
+    auto exps = [&](int i) {
+        if constexpr (kJoint) {
+            split_joint_exp(b[i][0], b[i][1], m0[i], m1[i]);
+            jt.term(split_mag(a[i][0]), m0[i]);
+            jt.term(split_mag(a[i][1]), m1[i]);
+        } else {
+            ma = max(ma, max(split_mag(a[i][0]), split_mag(a[i][1])));
+            mb = max(mb, max(split_mag(b[i][0]), split_mag(b[i][1])));
+        }
+    };
+    if constexpr (kKeep) {
+#pragma unroll
+        for (int s = 0; s < KS; ++s)
+            if (s < ks) exps(s);
+    } else {
+        for (int s = 0; s < ks; ++s) {
+            load(s, 0);
+            exps(0);
+        }
+    }
+    if constexpr (kJoint) {
         rbad = jt.finish();
         ea = jt.ea;
     } else {
-        for (int s = 0; s < ks; ++s) {
-            load(s);
-            m0 = max(m0, max(split_mag(a0), split_mag(a1)));
-            m1 = max(m1, max(split_mag(b0), split_mag(b1)));
-        }
-        m0 = split_max4(m0);
-        m1 = split_max4(m1);
-        rbad = split_unsafe(m0);
-        cbad = split_unsafe(m1);
-        ea = split_exp(m0);
-        eb = split_exp(m1);
+        ma = split_max4(ma);
+        mb = split_max4(mb);
+        rbad = split_unsafe(ma);
+        cbad = split_unsafe(mb);
+        ea = split_exp(ma);
+        eb = split_exp(mb);
     }
     SplitCut ca, cb;
     SplitAcc acc;
@@ -279,30 +331,37 @@ __device__ __forceinline__ void split_tile(int ks, LA la, LB lb, bool same, z2 (
 #pragma unroll
             for (int d = 0; d < kSplitDigits; ++d) sum[j][d] = 0;
     }
-#pragma unroll 1
-    for (int s = 0; s < ks; ++s) {
-        if constexpr (KS > 1) {
-            load(s);
-            if constexpr (kJoint) split_joint_exp(b0, b1, m0, m1);
-        }
+    auto step = [&](int i) {
         if constexpr (kJoint) {
             // b is cut on the grid of c_k, a on that of 2^(ea - c_k)
-            const int c0 = split_exp(m0), c1 = split_exp(m1);
-            split_cut(ca, a0, a1, ea - c0, ea - c1);
-            split_cut(cb, b0, b1, c0, c1);
+            const int c0 = split_exp(m0[i]), c1 = split_exp(m1[i]);
+            split_cut(ca, a[i][0], a[i][1], ea - c0, ea - c1);
+            split_cut(cb, b[i][0], b[i][1], c0, c1);
         } else {
-            split_cut(ca, a0, a1, ea, ea);
+            split_cut(ca, a[i][0], a[i][1], ea, ea);
             if (same) cb = ca;
-            else split_cut(cb, b0, b1, eb, eb);
+            else split_cut(cb, b[i][0], b[i][1], eb, eb);
         }
         split_mma<KIND>(ca, cb, acc);
-        if constexpr (KS > 4) {
-            if ((s & 3) == 3) {     // 64 terms: what FP32 holds exactly
+    };
+    if constexpr (kKeep) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
+        for (int s = 0; s < KS; ++s)
+            if (s < ks) step(s);
+    } else {
+#pragma unroll 1
+        for (int s = 0; s < ks; ++s) {
+            load(s, 0);
+            if constexpr (kJoint) split_joint_exp(b[0][0], b[0][1], m0[0], m1[0]);
+            step(0);
+            if constexpr (KS > 4) {
+                if ((s & 3) == 3) {     // 64 terms: what FP32 holds exactly
 #pragma unroll
-                    for (int d = 0; d < kSplitDigits; ++d) sum[j][d] += __float2int_rn(acc[d][j]);
-                split_start(acc, 0.f);
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int d = 0; d < kSplitDigits; ++d) sum[j][d] += __float2int_rn(acc[d][j]);
+                    split_start(acc, 0.f);
+                }
             }
         }
     }
@@ -344,6 +403,48 @@ __device__ __forceinline__ void split_tile(int ks, LA la, LB lb, bool same, z2 (
             }
         }
     }
+}
+
+// split_tile for operands that are on their grids already: v[j] in units of
+// 2^(Ea + Eb - 54).
+template <SplitKind KIND, int KS, class LA, class LB>
+__device__ __forceinline__ void split_tile_on(int ks, LA la, LB lb, bool same, z2 (&v)[2]) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    SplitCut ca, cb;
+    SplitAcc acc;
+    int sum[4][kSplitDigits];
+    split_start(acc, 0.f);
+    if constexpr (KS > 4) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int d = 0; d < kSplitDigits; ++d) sum[j][d] = 0;
+    }
+#pragma unroll 1
+    for (int s = 0; s < ks; ++s) {
+        split_cut_on(ca, la(g, 8 * s + 2 * t), la(g, 8 * s + 2 * t + 1));
+        if (same) cb = ca;
+        else split_cut_on(cb, lb(g, 8 * s + 2 * t), lb(g, 8 * s + 2 * t + 1));
+        split_mma<KIND>(ca, cb, acc);
+        if constexpr (KS > 4) {
+            if ((s & 3) == 3) {     // 64 terms: what FP32 holds exactly
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int d = 0; d < kSplitDigits; ++d) sum[j][d] += __float2int_rn(acc[d][j]);
+                split_start(acc, 0.f);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int d = 0; d < kSplitDigits; ++d) {
+            if constexpr (KS <= 4) sum[j][d] = __float2int_rn(acc[d][j]);
+            else sum[j][d] += __float2int_rn(acc[d][j]);
+        }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) v[j] = zmk(split_value<false>(sum[j]), split_value<false>(sum[j + 2]));
 }
 
 }  // namespace crs

@@ -79,7 +79,9 @@ __global__ void __launch_bounds__(256) k_solve_tail(const __grid_constant__ Tail
     }
 }
 
-int tail_blocks(int m) { return m <= 4 ? 8 : (m <= 8 ? 4 : (m <= 16 ? 2 : 1)); }
+// Above m = 32 a level is long enough for its launch not to matter, and the level
+// kernels take more threads.
+int tail_blocks(int m) { return m <= 4 ? 8 : (m <= 8 ? 4 : (m <= 16 ? 2 : (m <= 32 ? 1 : 0))); }
 
 static cudaError_t launch_tail(void (*kernel)(TailArgs), dim3 grid, size_t smem, const TailArgs &ta, cudaStream_t s) {
     cudaLaunchAttribute at[2] = {};
@@ -104,11 +106,11 @@ static cudaError_t launch_tail(void (*kernel)(TailArgs), dim3 grid, size_t smem,
         case 8: k = split ? kernel<8, true> : kernel<8, false>; break;           \
         case 16: k = split ? kernel<16, true> : kernel<16, false>; break;        \
         case 32: k = kernel<32, true>; break;                                    \
-        case 64: k = kernel<64, true>; break;                                    \
         default: return cudaErrorInvalidValue;                                   \
     }
 
 cudaError_t prepare_tail(int m, int smem_optin) {
+    if (tail_blocks(m) == 0) return cudaSuccess;
     const int mt = pick_mt(m);
     const bool split = split_form(m, 8);
     void (*k)(TailArgs) = nullptr;
