@@ -1,5 +1,8 @@
-// cr_core.cuh -- the per-level steps of classic cyclic reduction in FP64, as
-// device functions that one CTA runs on one chunk of a level.
+// cr_core.cuh -- the per-level steps of classic cyclic reduction by FMAs, as
+// device functions that one CTA runs on one chunk of a level: FP64 blocks of
+// m <= 6 and m = 9, 10 and the FP32 levels of the mixed form.  The other FP64
+// blocks have the forms of cr_core64.cuh, with the same chunks, outputs and
+// boundary rules (see split_form).
 //
 // One level (Sec. 2, eq. Formulas; 0-based: odd block t at position 2t, even
 // block j at 2j+1, so odd t has the even blocks j = t-1 on its left and
@@ -223,7 +226,7 @@ __device__ __forceinline__ void chol_lower_wide(const LevelArgsT<R> &a, int64_t 
 }
 
 // Blocked forward substitution Z := L^{-1} Z for every column of every block
-// of a chunk, run by the whole CTA (used for MT >= 32, where a column-by-
+// of a chunk, run by the whole CTA (used for MT = 32 in FP32, where a column-by-
 // column substitution would be one long dependent chain per thread).  Rows
 // are taken in blocks of 16: the diagonal block is solved per column (a
 // chain of <= 16 rows), then the rows below are updated in parallel, one
@@ -257,8 +260,8 @@ __device__ __forceinline__ void trsm_lower_cta(const C *sL, const R *sInv, C *ba
                     ld_ = ld2;
                 }
             }
-            if constexpr (sizeof(R) == 4) {
-                // FP32 (latency-bound): the column's rows rb .. re-1 in
+            {
+                // latency-bound: the column's rows rb .. re-1 in
                 // registers, so the chain waits on FMAs, not on shared memory
                 C zr[BS];
 #pragma unroll
@@ -277,12 +280,6 @@ __device__ __forceinline__ void trsm_lower_cta(const C *sL, const R *sInv, C *ba
 #pragma unroll
                 for (int i = 0; i < BS; ++i)
                     if (i < nbr) z[(rb + i) * ld_] = zr[i];
-            } else {
-                for (int r = rb; r < re; ++r) {
-                    C acc = z[r * ld_];
-                    for (int s = rb; s < r; ++s) zmsub(acc, Lb[tri(r, s)], z[s * ld_]);
-                    z[r * ld_] = zscale(acc, ivb[r]);
-                }
             }
         }
         __syncthreads();
@@ -327,7 +324,7 @@ __device__ __forceinline__ void trsm_lower_h_cta(const C *sL, const R *sInv, C *
             const C *Lb = sL + b * TRI;
             const R *ivb = sInv + b * MT;
             C *z = base + b * bstride + col;
-            if constexpr (sizeof(R) == 4) {
+            {
                 C zr[BS];
 #pragma unroll
                 for (int i = 0; i < BS; ++i)
@@ -345,12 +342,6 @@ __device__ __forceinline__ void trsm_lower_h_cta(const C *sL, const R *sInv, C *
 #pragma unroll
                 for (int i = 0; i < BS; ++i)
                     if (i < nbr) z[(rb + i) * ld] = zr[i];
-            } else {
-                for (int r = re - 1; r >= rb; --r) {
-                    C acc = z[r * ld];
-                    for (int s = r + 1; s < re; ++s) zmsub_ca(acc, Lb[tri(s, r)], z[s * ld]);
-                    z[r * ld] = zscale(acc, ivb[r]);
-                }
             }
         }
         __syncthreads();
@@ -761,14 +752,10 @@ __device__ __forceinline__ void factor_chunk(const LevelArgsT<R> &a, int64_t chu
                         const int r = ke + rr, q = ke + qq;
                         C *Lb = sL + b * TRI;
                         C u = Lb[tri(r, q)];
-                        if constexpr (sizeof(R) == 4) {
-                            const C *Lr = Lb + tri(r, kb), *Lq = Lb + tri(q, kb);
+                        const C *Lr = Lb + tri(r, kb), *Lq = Lb + tri(q, kb);
         #pragma unroll
-                            for (int j = 0; j < 16; ++j)
-                                if (kb + j < ke) zmsub_cb(u, Lr[j], Lq[j]);
-                        } else {
-                            for (int s = kb; s < ke; ++s) zmsub_cb(u, Lb[tri(r, s)], Lb[tri(q, s)]);
-                        }
+                        for (int j = 0; j < 16; ++j)
+                            if (kb + j < ke) zmsub_cb(u, Lr[j], Lq[j]);
                         Lb[tri(r, q)] = u;
                     }
                     __syncthreads();

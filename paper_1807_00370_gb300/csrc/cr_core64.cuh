@@ -26,9 +26,10 @@ namespace crs {
 // Which blocks take these forms: those that fill their tiles well enough.  A
 // block of m <= 4 would fill a quarter of a fragment; at m = 5 the padding to
 // 8 x 8 costs more than the FMAs (factor and solve at N = 100003, k = 3: 815 + 1076
-// against 595 + 800 us), and so does that of m = 9 .. 11 to 16 x 16 (factor at
-// m = 9, N = 65842: 2602 against 1761 us; at m = 12, N = 27776: 1432 against 1622).
-__host__ __device__ constexpr bool split_form(int m, size_t rsize) { return rsize == 8 && (m >= 12 || m == 7 || m == 8); }
+// against 595 + 800 us), and so does that of m = 9 and 10 to 16 x 16 (factor at
+// m = 10, N = 48000: about 1900 against 1733 us; at m = 11, N = 36062: 1574 against
+// 1652, solve with k = 4 1009 against 1436).
+__host__ __device__ constexpr bool split_form(int m, size_t rsize) { return rsize == 8 && (m >= 11 || m == 7 || m == 8); }
 // The classes that have blocks of either kind.
 template <int MT, class R> struct Forms {
     static constexpr bool split = sizeof(R) == 8 && MT >= 8;
@@ -766,8 +767,8 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
     const int lane = tid & 31, g = lane >> 2, tq = lane & 3, warp = tid >> 5, nw = NT >> 5;
     const int g8 = (FULL || KS == 1) ? KS : (m + 7) >> 3, ncg = (kw + 7) >> 3, per = g8 * ncg;
 
-    for (int e = warp; e < nbh * per; e += nw) {
-        const int b = e / per, rem = e - b * per, R = rem / ncg, n0 = 8 * (rem - R * ncg);
+    // r of rows 8 R .. and columns n0 .. of block b
+    auto r_task = [&](int b, int R, int n0) {
         const int64_t t = t0 + b, yo = 2 * t * mk + cb + n0, xo = t * mm + 8 * R * m;
         const int nc = kw - n0;
         z2 v[2];
@@ -787,55 +788,180 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
             const int64_t o = t * mk + r * k + cb + n0 + g;
             if (CRS_IN(a, kDbgR, o)) a.r[o] = w;
         }
-    }
-    __syncthreads();
-    for (int pass = 0; pass < 2; ++pass) {      // 0: P^H r, 1: Q^H r
-        for (int e = warp; e < nbh * per; e += nw) {
-            const int b = e / per, rem = e - b * per, G = rem / ncg, n0 = 8 * (rem - G * ncg);
+    };
+    // Entry (p, n) of P^H r: kept in sW, or for the chunk's first block given to
+    // the previous chunk.
+    auto put_pr = [&](int b, int p, int n, z2 w) {
+        const int64_t t = t0 + b, rem = (int64_t)p * k + cb + n;
+        if (b > 0) {
+            sW[(b * MT + p) * kc + n] = w;
+        } else if (a.inline_fix) {
+            const int64_t o = (t - 1) * mk + rem;
+            if (CRS_IN(a, kDbgYn, o)) a.yn[o] = zsub(a.yn[o], w);
+        } else if (CRS_IN(a, kDbgCbd, chunk * mk + rem)) {
+            a.cbd[chunk * mk + rem] = w;
+        }
+    };
+    // v from y_even - Q^H r
+    auto put_v = [&](int b, int p, int n, z2 w) {
+        const int64_t o = (t0 + b) * mk + (int64_t)p * k + cb + n;
+        if (b + 1 < nbh) w = zsub(w, sW[((b + 1) * MT + p) * kc + n]);
+        if (CRS_IN(a, kDbgYn, o)) a.yn[o] = w;
+    };
+    auto load_y = [&](int b, int p, int n) {     // y_even, ahead of the product
+        const int64_t o = (2 * (t0 + b) + 1) * mk + (int64_t)p * k + cb + n;
+        return ((FULL || p < m) && n < kw && 2 * (t0 + b) + 1 < a.Nl && CRS_IN(a, kDbgY, o)) ? a.y[o] : zero;
+    };
+    // rows 8 G .. of P^H r (pass 0) or Q^H r (pass 1); keep: y_even - Q^H r goes to
+    // sR in the place of r
+    auto u_task = [&](int b, int pass, int G, int n0, bool keep) {
             const int64_t t = t0 + b, zo = t * m2 * m + (pass ? m : 0) + 8 * G;
-            if (pass ? 2 * t + 1 >= a.Nl : t < 1) continue;
+            if (pass ? 2 * t + 1 >= a.Nl : t < 1) return;
             const int nc = kw - n0, np = m - 8 * G;
             const z2 *Rb = sR + b * MT * kc + n0;
             z2 v[2], u[2];
             int ex[2];
-            if (pass) {     // y_even, loaded ahead of the product
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const int64_t oy = (2 * t + 1) * mk + (int64_t)(8 * G + g) * k + cb + n0 + 2 * tq + j;
-                    u[j] = ((FULL || g < np) && 2 * tq + j < nc && CRS_IN(a, kDbgY, oy)) ? a.y[oy] : zero;
-                }
-            }
+            for (int j = 0; j < 2; ++j) u[j] = pass ? load_y(b, 8 * G + g, n0 + 2 * tq + j) : zero;
             split_tile<kConjA, false, KS>(
                 g8,
                 [&](int i, int s) { return ((FULL || (i < np && s < m)) && CRS_IN(a, kDbgZ, zo + s * m2 + i)) ? a.Z[zo + s * m2 + i] : zero; },
                 [&](int i, int s) { return (i < nc && (FULL || s < m)) ? Rb[s * kc + i] : zero; }, false, v, ex);
+            if (keep) __syncwarp();     // sR is read up to here
             const int p = 8 * G + g;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 const int n = 2 * tq + j;
                 if ((!FULL && p >= m) || n >= nc) continue;
-                const int64_t rem2 = (int64_t)p * k + cb + n0 + n;
                 if (pass == 0) {
-                    const z2 w = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
-                    if (b > 0) {
-                        sW[(b * MT + p) * kc + n0 + n] = w;
-                    } else if (a.inline_fix) {
-                        const int64_t o = (t - 1) * mk + rem2;
-                        if (CRS_IN(a, kDbgYn, o)) a.yn[o] = zsub(a.yn[o], w);
-                    } else if (CRS_IN(a, kDbgCbd, chunk * mk + rem2)) {
-                        a.cbd[chunk * mk + rem2] = w;
-                    }
+                    put_pr(b, p, n0 + n, zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j])));
                 } else {
-                    z2 w = u[j];
                     const double sc = -split_scale(ex[j]);
-                    w.x = fma(v[j].x, sc, w.x);
-                    w.y = fma(v[j].y, sc, w.y);
-                    if (b + 1 < nbh) w = zsub(w, sW[((b + 1) * MT + p) * kc + n0 + n]);
-                    if (CRS_IN(a, kDbgYn, t * mk + rem2)) a.yn[t * mk + rem2] = w;
+                    const z2 w = zmk(fma(v[j].x, sc, u[j].x), fma(v[j].y, sc, u[j].y));
+                    if (keep) sR[(b * MT + p) * kc + n0 + n] = w;
+                    else put_v(b, p, n0 + n, w);
+                }
+            }
+    };
+
+    if constexpr (MT == 8) {
+        // One warp per block and 8 columns: all operands loaded at once, r stays
+        // in the lanes that need it for Z^H r; the same numbers as the tasks.
+        constexpr unsigned kAll = 0xffffffffu;
+        for (int e = warp; e < nbh * ncg; e += nw) {
+            const int b = e / ncg, n0 = 8 * (e - b * ncg);
+            const int64_t t = t0 + b;
+            const bool hasL = t >= 1, hasR = 2 * t + 1 < a.Nl;
+            const int nc = kw - n0;
+            z2 x[2], y[2], z[2][2], u[2], r[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int s = 2 * tq + j;
+                const int64_t oy = 2 * t * mk + (int64_t)s * k + cb + n0 + g, ox = t * mm + g * m + s, oz = t * m2 * m + s * m2 + g;
+                y[j] = (g < nc && (FULL || s < m) && CRS_IN(a, kDbgY, oy)) ? a.y[oy] : zero;
+                x[j] = ((FULL || g < m) && s <= g && CRS_IN(a, kDbgL, ox)) ? a.L[ox] : zero;
+                z[0][j] = (hasL && (FULL || (g < m && s < m)) && CRS_IN(a, kDbgZ, oz)) ? a.Z[oz] : zero;
+                z[1][j] = (hasR && (FULL || (g < m && s < m)) && CRS_IN(a, kDbgZ, oz + m)) ? a.Z[oz + m] : zero;
+                u[j] = load_y(b, g, n0 + s);
+            }
+            unsigned mx[2], mz[2];
+            SplitJoint jt;
+            split_joint_exp(x[0], x[1], mx[0], mx[1]);
+            jt.term(split_mag(y[0]), mx[0]);
+            jt.term(split_mag(y[1]), mx[1]);
+            bool ok = !jt.finish() && jt.ea >= kSplitSumTiny;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                mz[h] = split_max4(max(split_mag(z[h][0]), split_mag(z[h][1])));
+                if (split_unsafe(mz[h]) || split_exp(mz[h]) < kSplitSumTiny / 2) ok = false;
+            }
+            SplitCut c1, c2;
+            SplitAcc acc;
+            {
+                const int e0 = split_exp(mx[0]), e1 = split_exp(mx[1]);
+                split_cut(c1, y[0], y[1], jt.ea - e0, jt.ea - e1);
+                split_cut(c2, x[0], x[1], e0, e1);
+                split_start(acc, kSplitStart);
+                split_mma<kPlain>(c1, c2, acc);
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                int s0[kSplitDigits], s1[kSplitDigits];
+#pragma unroll
+                for (int d = 0; d < kSplitDigits; ++d) {
+                    s0[d] = __float_as_int(acc[d][j]);
+                    s1[d] = __float_as_int(acc[d][j + 2]);
+                }
+                r[j] = zmk(split_scaled(split_value<true>(s0), jt.ea), split_scaled(split_value<true>(s1), jt.ea));
+            }
+            const unsigned mr = split_max4(max(split_mag(r[0]), split_mag(r[1])));
+            const int er = split_exp(mr);
+            if (split_unsafe(mr) || er < kSplitSumTiny / 2) ok = false;
+            if (!__all_sync(kAll, ok)) {        // out of the split's range somewhere
+                r_task(b, 0, n0);
+                __syncwarp();
+                u_task(b, 0, 0, n0, false);
+                __syncwarp();
+                u_task(b, 1, 0, n0, true);
+                continue;
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int64_t o = t * mk + (int64_t)(2 * tq + j) * k + cb + n0 + g;
+                if (g < nc && (FULL || 2 * tq + j < m) && CRS_IN(a, kDbgR, o)) a.r[o] = r[j];
+            }
+            split_cut(c2, r[0], r[1], er, er);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h ? !hasR : !hasL) continue;
+                const int ez = split_exp(mz[h]);
+                split_cut(c1, z[h][0], z[h][1], ez, ez);
+                split_start(acc, kSplitStart);
+                split_mma<kConjA>(c1, c2, acc);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int ex = ez + __shfl_sync(kAll, er, 8 * tq + 4 * j), n = 2 * tq + j;
+                    int s0[kSplitDigits], s1[kSplitDigits];
+#pragma unroll
+                    for (int d = 0; d < kSplitDigits; ++d) {
+                        s0[d] = __float_as_int(acc[d][j]);
+                        s1[d] = __float_as_int(acc[d][j + 2]);
+                    }
+                    const z2 v = zmk(split_value<true>(s0), split_value<true>(s1));
+                    if ((!FULL && g >= m) || n >= nc) continue;
+                    if (h == 0) {
+                        put_pr(b, g, n0 + n, zmk(split_scaled(v.x, ex), split_scaled(v.y, ex)));
+                    } else {
+                        const double sc = -split_scale(ex);
+                        sR[(b * MT + g) * kc + n0 + n] = zmk(fma(v.x, sc, u[j].x), fma(v.y, sc, u[j].y));
+                    }
                 }
             }
         }
         __syncthreads();
+        for (int e = warp; e < nbh * ncg; e += nw) {
+            const int b = e / ncg, n0 = 8 * (e - b * ncg);
+            if (2 * (t0 + b) + 1 >= a.Nl) continue;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int n = n0 + 2 * tq + j;
+                if ((FULL || g < m) && n < kw) put_v(b, g, n, sR[(b * MT + g) * kc + n]);
+            }
+        }
+        __syncthreads();
+    } else {
+        for (int e = warp; e < nbh * per; e += nw) {
+            const int b = e / per, rem = e - b * per, R = rem / ncg;
+            r_task(b, R, 8 * (rem - R * ncg));
+        }
+        __syncthreads();
+        for (int pass = 0; pass < 2; ++pass) {      // 0: P^H r, 1: Q^H r
+            for (int e = warp; e < nbh * per; e += nw) {
+                const int b = e / per, rem = e - b * per, G = rem / ncg;
+                u_task(b, pass, G, 8 * (rem - G * ncg), false);
+            }
+            __syncthreads();
+        }
     }
     if (a.bd_count) {
         // counters of this right-hand-side chunk: [cchunk][boundary]
@@ -865,7 +991,8 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
     const int g8 = (FULL || KS == 1) ? KS : (m + 7) >> 3, ncg = (kw + 7) >> 3, per = g8 * ncg;
 
     const bool failed = a.level == 0 && *a.status != CRS_NO_FAIL;   // the result is NaN
-    for (int e = tid; e < nbh * m * kw; e += NT) {
+    // the even unknowns (MT = 8: below, with the lanes' operands)
+    for (int e = tid; e < ((MT > 8 || failed) ? nbh * m * kw : 0); e += NT) {
         const int b = e / (m * kw), rem = e - b * (m * kw), r = rem / kw, c = rem - r * kw;
         const int64_t t = t0 + b, o = (int64_t)r * k + cb + c;
         if (failed && CRS_IN(a, kDbgX, 2 * t * mk + o)) a.x[2 * t * mk + o] = zmk(qnan(0.0), qnan(0.0));
@@ -875,8 +1002,7 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
     }
     if (failed) return;
 
-    for (int e = warp; e < nbh * per; e += nw) {
-        const int b = e / per, rem = e - b * per, R = rem / ncg, n0 = 8 * (rem - R * ncg);
+    auto w_task = [&](int b, int R, int n0) {
         const int64_t t = t0 + b, zo = t * m2 * m + 8 * R * m2;
         const int nc = kw - n0;
         const bool hasL = t >= 1, hasR = t < a.ne;
@@ -913,10 +1039,8 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
             w.y = fma(v[j].y, sc, w.y);
             sW[(b * MT + r) * kc + n0 + g] = w;
         }
-    }
-    __syncthreads();
-    for (int e = warp; e < nbh * per; e += nw) {
-        const int b = e / per, rem = e - b * per, G = rem / ncg, n0 = 8 * (rem - G * ncg);
+    };
+    auto x_task = [&](int b, int G, int n0) {
         const int64_t t = t0 + b, xo = t * mm + 8 * G * m + 8 * G;
         const int nc = kw - n0, np = m - 8 * G;
         const z2 *Wb = sW + (b * MT + 8 * G) * kc + n0;
@@ -932,6 +1056,101 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
             const int64_t o = 2 * t * mk + (int64_t)p * k + cb + n0 + n;
             if ((FULL || p < m) && n < nc && CRS_IN(a, kDbgX, o))
                 a.x[o] = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
+        }
+    };
+
+    if constexpr (MT == 8) {
+        // One warp per block and 8 columns, as in the down sweep.
+        constexpr unsigned kAll = 0xffffffffu;
+        for (int e = warp; e < nbh * ncg; e += nw) {
+            const int b = e / ncg, n0 = 8 * (e - b * ncg);
+            const int64_t t = t0 + b;
+            const int nc = kw - n0;
+            z2 xn[2][2], z[2][2], x[2], w[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int s = 2 * tq + j;
+                const bool in = FULL || (g < m && s < m);
+                const int64_t o = t * mk + (int64_t)s * k + cb + n0 + g, oz = t * m2 * m + g * m2 + s, ox = t * mm + s * m + g;
+                const bool col = g < nc && (FULL || s < m);
+                xn[0][j] = (col && t >= 1 && CRS_IN(a, kDbgXn, o - mk)) ? a.xn[o - mk] : zero;
+                xn[1][j] = (col && t < a.ne && CRS_IN(a, kDbgXn, o)) ? a.xn[o] : zero;
+                w[j] = (col && CRS_IN(a, kDbgR, o)) ? a.r[o] : zero;
+                z[0][j] = (in && CRS_IN(a, kDbgZ, oz)) ? a.Z[oz] : zero;
+                z[1][j] = (in && CRS_IN(a, kDbgZ, oz + m)) ? a.Z[oz + m] : zero;
+                x[j] = (in && g <= s && CRS_IN(a, kDbgL, ox)) ? a.L[ox] : zero;
+                const int64_t oe = (2 * t + 1) * mk + (int64_t)s * k + cb + n0 + g;
+                if (col && t < a.ne && CRS_IN(a, kDbgX, oe)) a.x[oe] = xn[1][j];
+            }
+            unsigned mx[2][2];
+            SplitJoint jt;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                split_joint_exp(z[h][0], z[h][1], mx[h][0], mx[h][1]);
+                jt.term(split_mag(xn[h][0]), mx[h][0]);
+                jt.term(split_mag(xn[h][1]), mx[h][1]);
+            }
+            bool ok = !jt.finish() && jt.ea >= kSplitSumTiny;
+            const unsigned ml = split_max4(max(split_mag(x[0]), split_mag(x[1])));
+            if (split_unsafe(ml) || split_exp(ml) < kSplitSumTiny / 2) ok = false;
+            SplitCut c1, c2;
+            SplitAcc acc;
+            split_start(acc, 0.f);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int e0 = split_exp(mx[h][0]), e1 = split_exp(mx[h][1]);
+                split_cut(c1, xn[h][0], xn[h][1], jt.ea - e0, jt.ea - e1);
+                split_cut(c2, z[h][0], z[h][1], e0, e1);
+                split_mma<kPlain>(c1, c2, acc);
+            }
+            const double sc = -split_scale(jt.ea);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                int s0[kSplitDigits], s1[kSplitDigits];
+#pragma unroll
+                for (int d = 0; d < kSplitDigits; ++d) {
+                    s0[d] = __float2int_rn(acc[d][j]);
+                    s1[d] = __float2int_rn(acc[d][j + 2]);
+                }
+                w[j].x = fma(split_value<false>(s0), sc, w[j].x);
+                w[j].y = fma(split_value<false>(s1), sc, w[j].y);
+            }
+            const unsigned mw = split_max4(max(split_mag(w[0]), split_mag(w[1])));
+            const int ew = split_exp(mw), el = split_exp(ml);
+            if (split_unsafe(mw) || ew < kSplitSumTiny / 2) ok = false;
+            if (!__all_sync(kAll, ok)) {        // out of the split's range somewhere
+                w_task(b, 0, n0);
+                __syncwarp();
+                x_task(b, 0, n0);
+                continue;
+            }
+            split_cut(c1, x[0], x[1], el, el);
+            split_cut(c2, w[0], w[1], ew, ew);
+            split_start(acc, kSplitStart);
+            split_mma<kConjA>(c1, c2, acc);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int ex = el + __shfl_sync(kAll, ew, 8 * tq + 4 * j), n = 2 * tq + j;
+                int s0[kSplitDigits], s1[kSplitDigits];
+#pragma unroll
+                for (int d = 0; d < kSplitDigits; ++d) {
+                    s0[d] = __float_as_int(acc[d][j]);
+                    s1[d] = __float_as_int(acc[d][j + 2]);
+                }
+                const int64_t o = 2 * t * mk + (int64_t)g * k + cb + n0 + n;
+                if ((FULL || g < m) && n < nc && CRS_IN(a, kDbgX, o))
+                    a.x[o] = zmk(split_scaled(split_value<true>(s0), ex), split_scaled(split_value<true>(s1), ex));
+            }
+        }
+    } else {
+        for (int e = warp; e < nbh * per; e += nw) {
+            const int b = e / per, rem = e - b * per, R = rem / ncg;
+            w_task(b, R, 8 * (rem - R * ncg));
+        }
+        __syncthreads();
+        for (int e = warp; e < nbh * per; e += nw) {
+            const int b = e / per, rem = e - b * per, G = rem / ncg;
+            x_task(b, G, 8 * (rem - G * ncg));
         }
     }
 }

@@ -87,8 +87,7 @@ __global__ void __launch_bounds__(256) k_solve_up_wide(LevelArgsT<R> a) {
 }
 
 // The split forms of the FP64 levels (cr_core64.cuh).
-// Class 64: one CTA fits on an SM, which runs twice the tile's threads (level 0
-// of N = 4096, m = 64: 3957 us at 256, 3335 at 512).
+// (class 64 at twice the tile's threads: split_threads)
 template <int MT>
 __global__ void __launch_bounds__(MT == 64 ? 512 : 256) k_factor_split(LevelArgs a) {
     level_begin();
@@ -96,13 +95,13 @@ __global__ void __launch_bounds__(MT == 64 ? 512 : 256) k_factor_split(LevelArgs
     factor_chunk_split<MT>(a, a.c_begin + blockIdx.x, smem_raw);
 }
 template <int MT>
-__global__ void __launch_bounds__(256) k_solve_down_split(LevelArgs a) {
+__global__ void __launch_bounds__(256, MT <= 16 ? 2 : 0) k_solve_down_split(LevelArgs a) {
     level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_down_chunk_split<MT>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
 }
 template <int MT>
-__global__ void __launch_bounds__(256) k_solve_up_split(LevelArgs a) {
+__global__ void __launch_bounds__(256, MT <= 16 ? 2 : 0) k_solve_up_split(LevelArgs a) {
     level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve_up_chunk_split<MT>(a, a.c_begin + blockIdx.x, blockIdx.y, smem_raw);
@@ -471,13 +470,19 @@ static bool solve_wide(const LevelArgsT<R> &a) {
     return MT < 32 && narrowed && a.nb * a.kc <= kWideCols;
 }
 
+// Threads of the split factor for a tile of `th`: twice as many in class 64, where
+// one CTA fits on an SM (level 0 of N = 4096, m = 64: 3957 us at 256, 3335 at 512),
+// half in class 8, whose blocks take a warp each and leave the registers for
+// four CTAs of 128 (N = 2^18, m = 8, all levels: 1694 us at 256, 1522 at 128).
+static int split_threads(int mt, int th) { return mt == 64 ? 2 * th : (mt == 8 ? std::max(th / 64 * 32, 64) : th); }
+
 template <int MT, class R>
 static cudaError_t factor_odd_mt(const LevelArgsT<R> &a, cudaStream_t s) {
     const unsigned grid = odd_grid(a);
     const int th = sizeof(R) == 4 ? tile_shape32(MT).threads : tile_shape(MT).threads;
     if constexpr (Forms<MT, R>::split) {
         if (split_form(a.m, sizeof(R))) {
-            launch_level(k_factor_split<MT>, grid, MT == 64 ? 2 * th : th, a.nb * factor64_entries(MT) * sizeof(z2), s, a);
+            launch_level(k_factor_split<MT>, grid, split_threads(MT, th), a.nb * factor64_entries(MT) * sizeof(z2), s, a);
             return cudaGetLastError();
         }
     }
