@@ -172,10 +172,14 @@ int crsolve_set_scratch(crsolve_plan p, void *dev_ptr, size_t bytes);
  *   P_i = L_i^{-1} B_{i-1}, Q_i = L_i^{-1} B_i^H and the half-size even system
  *   V_j = A_{2j} - Q_{2j-1}^H Q_{2j-1} - P_{2j+1}^H P_{2j+1},
  *   F_j = -Q_{2j+1}^H P_{2j+1} (eq. Formulas with the Sec. 4 product rule),
- *   and keeps L, P, Q of every level in the workspace for later solves.
+ *   and keeps L (or its inverse, by block size), P, Q of every level in the
+ *   workspace for later solves.
  *   On a classic FP64 plan it enqueues only kernels and memsets on the
  *   stream: one kernel per level, plus a fix-up kernel for the CTA-boundary
- *   blocks on levels of more than four CTAs per SM.
+ *   blocks on levels of more than four CTAs per SM.  Systems of N < 8192 and
+ *   m <= 32 run their coarse levels in one kernel (and the solve's two sweeps of
+ *   them in another), counted and timed under the finest of these levels as
+ *   CRSOLVE_K_FACTOR_ODD and CRSOLVE_K_SOLVE_DOWN_ODD.
  * Returns CRSOLVE_OK once enqueued; breakdown is reported by crsolve_info_get.
  */
 int crsolve_factor(crsolve_plan p, const crsolve_z *A, const crsolve_z *B, void *stream);

@@ -1,10 +1,9 @@
 // cr_device.cuh -- device-side helpers shared by the cyclic-reduction kernels.
 //
 // Complex numbers are double2 (x = real, y = imaginary), the byte layout of
-// crsolve_z / complex128.  Every complex multiply-add is written as four
-// fused multiply-adds: on GB300 the FP64 pipe (2 DFMA per clock per SM) is the
-// bound of the whole FP64 path, so the kernels count FP64 instructions, not
-// bytes.
+// crsolve_z / complex128.  Every complex multiply-add here is written as four
+// fused multiply-adds: on GB300 the FP64 pipe (2 DFMA per clock per SM) bounds the
+// FMA forms of the FP64 path, so they count FP64 instructions, not bytes.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
