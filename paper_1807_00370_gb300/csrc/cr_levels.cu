@@ -219,7 +219,7 @@ __global__ void k_nan_if_failed(z2 *x, int64_t n, const unsigned long long *stat
 // N = 2^14, m = 64, k = 32); crsolve_tile_set overrides them.
 static TileShape g_tiles[5] = {
     {32, 32, 32, 256, 256},  // MT = 4
-    {16, 16, 16, 256, 128},  // MT = 8
+    {16, 8, 16, 256, 128},   // MT = 8
     {8, 4, 8, 256, 128},     // MT = 16
     {2, 1, 8, 256, 128},     // MT = 32
     {1, 1, 8, 256, 128},     // MT = 64
