@@ -104,23 +104,24 @@ __device__ inline void make_level_args(LevelArgs &a, const BatchArgs &ba, const 
     a.dbg = ba.dbg;
 }
 
-// One chunk in the form of its block size (the form the level kernels take).
+// One chunk in the form of its block size (the form the level kernels take); a
+// function each, which keeps the kernel quick to compile.
 template <int MT>
-__device__ __forceinline__ void factor_of(const LevelArgs &a, int64_t c, unsigned char *smem) {
+__device__ __noinline__ void factor_of(const LevelArgs &a, int64_t c, unsigned char *smem) {
     if constexpr (Forms<MT, double>::fma) {
         if (!split_form(a.m, 8)) return factor_chunk<MT, double>(a, c, smem);
     }
     if constexpr (Forms<MT, double>::split) factor_chunk_split<MT>(a, c, smem);
 }
 template <int MT>
-__device__ __forceinline__ void solve_down_of(const LevelArgs &a, int64_t c, int cc, unsigned char *smem) {
+__device__ __noinline__ void solve_down_of(const LevelArgs &a, int64_t c, int cc, unsigned char *smem) {
     if constexpr (Forms<MT, double>::fma) {
         if (!split_form(a.m, 8)) return solve_down_chunk<MT, double>(a, c, cc, smem);
     }
     if constexpr (Forms<MT, double>::split) solve_down_chunk_split<MT>(a, c, cc, smem);
 }
 template <int MT>
-__device__ __forceinline__ void solve_up_of(const LevelArgs &a, int64_t c, int cc, unsigned char *smem) {
+__device__ __noinline__ void solve_up_of(const LevelArgs &a, int64_t c, int cc, unsigned char *smem) {
     if constexpr (Forms<MT, double>::fma) {
         if (!split_form(a.m, 8)) return solve_up_chunk<MT, double>(a, c, cc, smem);
     }
