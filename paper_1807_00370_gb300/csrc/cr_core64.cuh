@@ -534,7 +534,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                         int sum[kSplitDigits];
 #pragma unroll
                         for (int d = 0; d < kSplitDigits; ++d) sum[d] = __float_as_int(acc[d][j]);
-                        v[j] = split_scaled(split_value<true>(sum), jt[h].ea);
+                        v[j] = split_scaled(split_value<1>(sum), jt[h].ea);
                     }
                     z[h][0] = zmk(v[0], v[2]);
                     z[h][1] = zmk(v[1], v[3]);
@@ -581,7 +581,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                             s0[d] = __float_as_int(acc[d][j]);
                             s1[d] = __float_as_int(acc[d][j + 2]);
                         }
-                        const z2 v = zmk(split_value<true>(s0), split_value<true>(s1));
+                        const z2 v = zmk(split_value<1>(s0), split_value<1>(s1));
                         if ((!FULL && (p >= m || q >= m)) || (f != 1 && q > p)) continue;
                         if (f == 2) {
                             Zb[p * LDZ + q] = sub_qq(load_a(b, p, q), p, q, v, ex);
@@ -892,7 +892,7 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
                     s0[d] = __float_as_int(acc[d][j]);
                     s1[d] = __float_as_int(acc[d][j + 2]);
                 }
-                r[j] = zmk(split_scaled(split_value<true>(s0), jt.ea), split_scaled(split_value<true>(s1), jt.ea));
+                r[j] = zmk(split_scaled(split_value<1>(s0), jt.ea), split_scaled(split_value<1>(s1), jt.ea));
             }
             const unsigned mr = split_max4(max(split_mag(r[0]), split_mag(r[1])));
             const int er = split_exp(mr);
@@ -927,7 +927,7 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
                         s0[d] = __float_as_int(acc[d][j]);
                         s1[d] = __float_as_int(acc[d][j + 2]);
                     }
-                    const z2 v = zmk(split_value<true>(s0), split_value<true>(s1));
+                    const z2 v = zmk(split_value<1>(s0), split_value<1>(s1));
                     if ((!FULL && g >= m) || n >= nc) continue;
                     if (h == 0) {
                         put_pr(b, g, n0 + n, zmk(split_scaled(v.x, ex), split_scaled(v.y, ex)));
@@ -1112,8 +1112,8 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
                     s0[d] = __float2int_rn(acc[d][j]);
                     s1[d] = __float2int_rn(acc[d][j + 2]);
                 }
-                w[j].x = fma(split_value<false>(s0), sc, w[j].x);
-                w[j].y = fma(split_value<false>(s1), sc, w[j].y);
+                w[j].x = fma(split_value<2>(s0), sc, w[j].x);
+                w[j].y = fma(split_value<2>(s1), sc, w[j].y);
             }
             const unsigned mw = split_max4(max(split_mag(w[0]), split_mag(w[1])));
             const int ew = split_exp(mw), el = split_exp(ml);
@@ -1139,7 +1139,7 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
                 }
                 const int64_t o = 2 * t * mk + (int64_t)g * k + cb + n0 + n;
                 if ((FULL || g < m) && n < nc && CRS_IN(a, kDbgX, o))
-                    a.x[o] = zmk(split_scaled(split_value<true>(s0), ex), split_scaled(split_value<true>(s1), ex));
+                    a.x[o] = zmk(split_scaled(split_value<1>(s0), ex), split_scaled(split_value<1>(s1), ex));
             }
         }
     } else {

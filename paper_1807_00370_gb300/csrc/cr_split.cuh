@@ -170,16 +170,25 @@ __device__ __forceinline__ void split_mma(const SplitCut &a, const SplitCut &b, 
     }
 }
 
-// The integer sum of a tile's digit products in units of 2^(Ea + Eb - 54 + kShift)
-// as a double, from the sums per digit (kMagic: each offset by kSplitMagic):
-// below 2^63 for up to 128 real terms, with kShift = 1 up to 256.
-template <bool kMagic, int kShift = 0>
-__device__ __forceinline__ double split_value(const int (&s)[kSplitDigits]) {
-    constexpr int H = kShift;
-    constexpr uint64_t M = kMagic ? (uint64_t)kSplitMagic : 0;
+// The integer sum of a tile's digit products over KS K-steps (16 KS real terms) as
+// a double, in units of 2^(Ea + Eb - 54), above 8 K-steps of 2^(Ea + Eb - 53), from
+// the sums per digit (KS = 1: each offset by kSplitMagic).  It is below 2^63 for up
+// to 128 real terms, in the larger unit up to 256.  A real term adds up to 196608 =
+// 2 * 512 * 128 + 4 * 128^2 to s[5] and 212992 to s[6]: 256 s[5] + s[6] stays below
+// 2^31 over the 32 terms of two K-steps, beyond it is formed in 64 bits.
+template <int KS>
+__host__ __device__ __forceinline__ double split_value(const int (&s)[kSplitDigits]) {
+    constexpr int H = KS > 8 ? 1 : 0;
+    constexpr uint64_t M = KS == 1 ? (uint64_t)kSplitMagic : 0;
     constexpr uint64_t off = (M << (38 - H)) + (M << (30 - H)) + (M << (22 - H)) + (M << (14 - H)) + (M << (6 - H));
-    const int low = (int)((uint32_t)s[5] * 256u + (uint32_t)s[6] + ((512u << H) - (uint32_t)(M * 257)));
-    uint64_t v = (uint64_t)(int64_t)(low >> (10 + H)) - off;
+    uint64_t v;
+    if constexpr (KS <= 2) {
+        const int low = (int)((uint32_t)s[5] * 256u + (uint32_t)s[6] + ((512u << H) - (uint32_t)(M * 257)));
+        v = (uint64_t)(int64_t)(low >> (10 + H)) - off;
+    } else {
+        const int64_t low = (int64_t)s[5] * 256 + s[6] + (512 << H);
+        v = (uint64_t)(low >> (10 + H));
+    }
     v += (uint64_t)((int64_t)s[4] * (1 << (6 - H)));
     v += (uint64_t)((int64_t)s[3] * (1 << (14 - H)));
     v += (uint64_t)((int64_t)s[2] * (1 << (22 - H)));
@@ -375,7 +384,7 @@ __device__ __forceinline__ void split_tile(int ks, LA la, LB lb, bool same, z2 (
         }
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-        v[j] = zmk(split_value<KS == 1, (KS > 8)>(sum[j]), split_value<KS == 1, (KS > 8)>(sum[j + 2]));
+        v[j] = zmk(split_value<KS>(sum[j]), split_value<KS>(sum[j + 2]));
         e[j] = ea + (kJoint ? 0 : __shfl_sync(kAll, eb, 8 * t + 4 * j)) + (KS > 8 ? 1 : 0);
     }
     if (__any_sync(kAll, rbad || cbad || min(e[0], e[1]) < kSplitSumTiny)) {
@@ -444,7 +453,7 @@ __device__ __forceinline__ void split_tile_on(int ks, LA la, LB lb, bool same, z
             else sum[j][d] += __float2int_rn(acc[d][j]);
         }
 #pragma unroll
-    for (int j = 0; j < 2; ++j) v[j] = zmk(split_value<false>(sum[j]), split_value<false>(sum[j + 2]));
+    for (int j = 0; j < 2; ++j) v[j] = zmk(split_value<(KS > 2 ? KS : 2)>(sum[j]), split_value<(KS > 2 ? KS : 2)>(sum[j + 2]));
 }
 
 }  // namespace crs
