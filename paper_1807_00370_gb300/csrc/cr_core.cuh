@@ -623,11 +623,11 @@ __device__ __forceinline__ void factor_chunk(const LevelArgsT<R> &a, int64_t chu
                     const int b = e / mm, rem = e - b * mm, r = rem / m, c = rem - r * m;
                     const int64_t t = t0 + b, pos = 2 * t;
                     if (r >= c) {
-                        if (CRS_IN(a, kDbgA, pos * mm + rem)) va[u] = __ldg(a.A + pos * mm + rem);
-                        if (t < a.ne && CRS_IN(a, kDbgA, (pos + 1) * mm + rem)) vv[u] = __ldg(a.A + (pos + 1) * mm + rem);
+                        if (CRS_IN(a, kDbgA, pos * mm + rem)) va[u] = ld_level(a.A + pos * mm + rem);
+                        if (t < a.ne && CRS_IN(a, kDbgA, (pos + 1) * mm + rem)) vv[u] = ld_level(a.A + (pos + 1) * mm + rem);
                     }
-                    if (pos >= 1 && CRS_IN(a, kDbgB, (pos - 1) * mm + rem)) vp[u] = __ldg(a.B + (pos - 1) * mm + rem);
-                    if (pos + 1 < a.Nl && CRS_IN(a, kDbgB, pos * mm + rem)) vq[u] = __ldg(a.B + pos * mm + rem);
+                    if (pos >= 1 && CRS_IN(a, kDbgB, (pos - 1) * mm + rem)) vp[u] = ld_level(a.B + (pos - 1) * mm + rem);
+                    if (pos + 1 < a.Nl && CRS_IN(a, kDbgB, pos * mm + rem)) vq[u] = ld_level(a.B + pos * mm + rem);
                 }
             }
 #pragma unroll
@@ -1106,7 +1106,7 @@ __device__ __forceinline__ void solve_down_chunk(const LevelArgsT<R> &a, int64_t
             for (int s = 0; s < MT; ++s)
                 if (s < m) {
                     const int64_t zo = t * (int64_t)(m * m2) + p + s * m2;
-                    const C z = CRS_IN(a, kDbgZ, zo) ? __ldg(Zt + s * m2) : zmk(R(0), R(0));
+                    const C z = CRS_IN(a, kDbgZ, zo) ? ld_level(Zt + s * m2) : zmk(R(0), R(0));
                     zmac_ca(acc, zmk(flip_if(z.x, sg), flip_if(z.y, sg)), Rb[s * kc]);
                 }
             *dst = acc;
@@ -1256,7 +1256,7 @@ __device__ __forceinline__ void solve_up_chunk(const LevelArgsT<R> &a, int64_t c
             const C *Zr = a.Z + t * (int64_t)(m * m2) + r * m2;
 #pragma unroll
             for (int s = 0; s < 2 * MT; ++s)
-                if (s < m2 && CRS_IN(a, kDbgZ, t * (int64_t)(m * m2) + r * m2 + s)) zmsub(acc, __ldg(Zr + s), Xb[s * kc]);
+                if (s < m2 && CRS_IN(a, kDbgZ, t * (int64_t)(m * m2) + r * m2 + s)) zmsub(acc, ld_level(Zr + s), Xb[s * kc]);
             sW[(b * MT + r) * kc + c] = acc;
         }
     }

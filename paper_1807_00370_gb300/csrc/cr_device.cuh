@@ -28,6 +28,13 @@ __device__ __forceinline__ void level_begin() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// A load of a level's array.  FP32 levels may load through the read-only path: their
+// kernels start after the ones before them have ended.  FP64 kernels are set up
+// ahead (level_begin), and the batched kernel writes what it reads, so there
+// the data change during the kernel's life and the load is a plain one.
+__device__ __forceinline__ float2 ld_level(const float2 *p) { return __ldg(p); }
+__device__ __forceinline__ double2 ld_level(const double2 *p) { return *p; }
+
 #define CRS_NO_FAIL 0xFFFFFFFFFFFFFFFFull
 
 __device__ __forceinline__ double fmx(double a, double b, double c) { return fma(a, b, c); }
