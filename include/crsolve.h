@@ -180,6 +180,15 @@ int crsolve_set_scratch(crsolve_plan p, void *dev_ptr, size_t bytes);
  *   m <= 32 run their coarse levels in one kernel (and the solve's two sweeps of
  *   them in another), counted and timed under the finest of these levels as
  *   CRSOLVE_K_FACTOR_ODD and CRSOLVE_K_SOLVE_DOWN_ODD.
+ *   Accuracy of the FP64 form: blocks of m <= 6 and m = 9, 10 use FMAs and
+ *   substitutions.  The products of the others are formed from 57-bit
+ *   fixed-point operands on the tensor cores and rounded once; a result much
+ *   smaller than its largest operands' product (modulus below 2^-8 of it, or a
+ *   real or imaginary part below 2^-14) that owes this to its own terms and not
+ *   to cancellation is formed by FMAs.  So an entry over K real terms is within
+ *   K 2^-45 of the sum of its terms' moduli (K 2^-39 for one part against its own
+ *   real products) if all errors add up, and typically within an ulp or two.
+ *   Magnitudes below 2^-1042 may count as zero.
  * Returns CRSOLVE_OK once enqueued; breakdown is reported by crsolve_info_get.
  */
 int crsolve_factor(crsolve_plan p, const crsolve_z *A, const crsolve_z *B, void *stream);

@@ -223,7 +223,6 @@ __device__ __forceinline__ void inverse_chunk(const LevelArgs &a, int64_t t0, z2
     } else {
         constexpr int SL = Split64<MT>::SL, SU = Split64<MT>::SC, KS = MT / 8;
         z2 *sU = sC;
-        const z2 zero = zmk(0.0, 0.0);
         const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, tq = lane & 3, warp = tid >> 5, nw = blockDim.x >> 5;
         const int g8 = FULL ? KS : (m + 7) >> 3;
         for (int J = 0; J <= g8; ++J) {
@@ -236,9 +235,10 @@ __device__ __forceinline__ void inverse_chunk(const LevelArgs &a, int64_t t0, z2
                 int ex[2];
                 if (f < nT) {
                     const int I = J + f;
-                    auto row = [&](int r, int k) { return (FULL || r < m) ? Lb[tri(r, k)] : zero; };
-                    split_tile<kConjB, false, KS>(J, [&](int i, int k) { return row(8 * I + i, k); },
-                                                  [&](int i, int k) { return row(8 * J + i, k); }, I == J, v, ex);
+                    auto row = [=](int R) {
+                        return [=](int i, int k) { return (FULL || 8 * R + i < m) ? Lb[tri(8 * R + i, k)] : zmk(0.0, 0.0); };
+                    };
+                    split_tile<kConjB, false, KS>(J, row(I), row(J), {m - 8 * I, m - 8 * J, I == J ? kGram : kFull}, I == J, v, ex);
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const int r = 8 * I + g, c = 8 * J + 2 * tq + j;
@@ -251,8 +251,8 @@ __device__ __forceinline__ void inverse_chunk(const LevelArgs &a, int64_t t0, z2
                 } else {
                     const int I = J - 1, K = f - nT;
                     const z2 *Ub = sU + b * SU + 8 * K;
-                    auto x = [&](int i, int k) { return (k <= i && (FULL || 8 * I + i < m)) ? Lb[tri(8 * I + i, 8 * I + k)] : zero; };
-                    split_tile<kPlain, true, 1>(1, [&](int i, int k) { return (FULL || 8 * I + k < m) ? Ub[k * MT + i] : zero; }, x, false, v, ex);
+                    auto x = [=](int i, int k) { return (k <= i && (FULL || 8 * I + i < m)) ? Lb[tri(8 * I + i, 8 * I + k)] : zmk(0.0, 0.0); };
+                    split_tile<kPlain, true, 1>(1, [=](int i, int k) { return (FULL || 8 * I + k < m) ? Ub[k * MT + i] : zmk(0.0, 0.0); }, x, {8, m - 8 * I, kFull}, false, v, ex);
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const int r = 8 * I + 2 * tq + j;
@@ -274,8 +274,8 @@ __device__ __forceinline__ void inverse_chunk(const LevelArgs &a, int64_t t0, z2
                 if (f < nL) {
                     const int I = J + 1 + f;
                     // block column J is complete (8 wide) as there is a row below it
-                    split_tile<kConjB, true, 1>(1, [&](int i, int k) { return (FULL || 8 * I + i < m) ? Lb[tri(8 * I + i, 8 * J + k)] : zero; },
-                                                [&](int i, int k) { return k <= i ? Lb[tri(8 * J + i, 8 * J + k)] : zero; }, false, v, ex);
+                    split_tile<kConjB, true, 1>(1, [=](int i, int k) { return (FULL || 8 * I + i < m) ? Lb[tri(8 * I + i, 8 * J + k)] : zmk(0.0, 0.0); },
+                                                [=](int i, int k) { return k <= i ? Lb[tri(8 * J + i, 8 * J + k)] : zmk(0.0, 0.0); }, {m - 8 * I, 8, kFull}, false, v, ex);
                     __syncwarp();
 #pragma unroll
                     for (int j = 0; j < 2; ++j)
@@ -285,11 +285,11 @@ __device__ __forceinline__ void inverse_chunk(const LevelArgs &a, int64_t t0, z2
                     const int K = f - nL;
                     split_tile<kPlain, false, KS>(
                         J - K,
-                        [&](int i, int k) {     // column i of X
+                        [=](int i, int k) {     // column i of X
                             const int r = 8 * K + k, c = 8 * K + i;
-                            return c <= r ? Lb[tri(r, c)] : zero;
+                            return c <= r ? Lb[tri(r, c)] : zmk(0.0, 0.0);
                         },
-                        [&](int i, int k) { return (FULL || 8 * J + i < m) ? Lb[tri(8 * J + i, 8 * K + k)] : zero; }, false, v, ex);
+                        [=](int i, int k) { return (FULL || 8 * J + i < m) ? Lb[tri(8 * J + i, 8 * K + k)] : zmk(0.0, 0.0); }, {8, m - 8 * J, kFull}, false, v, ex);
 #pragma unroll
                     for (int j = 0; j < 2; ++j)
                         if (FULL || 8 * J + 2 * tq + j < m)
@@ -344,15 +344,16 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
             for (int R = g8 - 1; R >= 0; --R) {
                 z2 v[2];
                 int ex[2];
+                const z2 *Zc = Zb + col - g, *XL = a.L;
                 split_tile<kPlain, true, KS>(
-                    R + 1, [&](int i, int k) { return (FULL || (i < nc && k < m)) ? Zb[k * LDZ + col - g + i] : zero; },
-                    [&](int i, int k) {
-                        if (!((FULL || 8 * R + i < m) && k <= 8 * R + i)) return zero;
+                    R + 1, [=](int i, int k) { return (FULL || (i < nc && k < m)) ? Zc[k * LDZ + i] : zmk(0.0, 0.0); },
+                    [=](int i, int k) {
+                        if (!((FULL || 8 * R + i < m) && k <= 8 * R + i)) return zmk(0.0, 0.0);
                         if constexpr (!kOn) return Xb[tri(8 * R + i, k)];
                         const int64_t o = t * mm + (8 * R + i) * m + k;     // (sL has X on its grid)
-                        return CRS_IN(a, kDbgL, o) ? a.L[o] : zero;
+                        return CRS_IN(a, kDbgL, o) ? XL[o] : zmk(0.0, 0.0);
                     },
-                    false, v, ex);
+                    {nc, m - 8 * R, kFull}, false, v, ex);
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
@@ -422,7 +423,8 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
     // kOn: the entries of X, B and Z are put on their grids once (see the end), with
     // the exponents of the block's columns in sE: those of X at 0, its rows at
     // MT, Z's at 2 MT (0: out of the split's range; the tile then takes Z as
-    // stored).  Pays from m > 16 on, where a tile's operands are read by many
+    // stored), and at 4 MT and 5 MT whether X's and Z's columns have imaginary
+    // parts.  Small results (split_needs) read the stored entries.  Pays from m > 16 on, where a tile's operands are read by many
     // tiles (level 0 of N = 4096, m = 64: 3335 -> 2884 us, m = 32: 448 -> 417;
     // N = 65536, m = 16: 1069 -> 1125).
     int *const sE = reinterpret_cast<int *>(sC);
@@ -448,27 +450,32 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
         for (int j = 0; j < 2; ++j) u[j] = pJ ? zero : load_a(b, 8 * I + g, 8 * J + 2 * tq + j);
         if constexpr (!kOn) {
             split_tile<kConjA, false, KS>(
-                g8, [&](int i, int k) { return (FULL || (i < ni && k < m)) ? zi[k * LDZ + i] : zero; },
-                [&](int i, int k) { return (FULL || (i < nj && k < m)) ? zj[k * LDZ + i] : zero; }, zi == zj, v, ex);
+                g8, [=](int i, int k) { return (FULL || (i < ni && k < m)) ? zi[k * LDZ + i] : zmk(0.0, 0.0); },
+                [=](int i, int k) { return (FULL || (i < nj && k < m)) ? zj[k * LDZ + i] : zmk(0.0, 0.0); }, {ni, nj, zi == zj ? kGram : kFull}, zi == zj, v, ex);
         } else {
             const int *ze = sE + b * SE + 2 * MT;
             const int ci = 8 * I + (pI ? 0 : m), cj = 8 * J + (pJ ? 0 : m);
             const int ei = (FULL || g < ni) ? ze[ci + g] : 1023, ej = (FULL || g < nj) ? ze[cj + g] : 1023;
-            if (__any_sync(0xffffffffu, ei < 600 || ej < 600)) {
-                const int64_t oz = t * m2 * m;
-                auto zg = [&](int c, int k) {
-                    const int64_t o = oz + k * m2 + c;
-                    return CRS_IN(a, kDbgZ, o) ? a.Z[o] : zero;
+            auto zg = [&](int c0, int nc) {
+                const int64_t oz = t * m2 * m + c0;
+                const z2 *Z = a.Z;
+                return [=](int i, int k) {
+                    const int64_t o = oz + k * m2 + i;
+                    return ((FULL || (i < nc && k < m)) && CRS_IN(a, kDbgZ, o)) ? Z[o] : zmk(0.0, 0.0);
                 };
-                split_tile<kConjA, false, KS>(
-                    g8, [&](int i, int k) { return (FULL || (i < ni && k < m)) ? zg(ci + i, k) : zero; },
-                    [&](int i, int k) { return (FULL || (i < nj && k < m)) ? zg(cj + i, k) : zero; }, zi == zj, v, ex);
+            };
+            auto zgi = zg(ci, ni), zgj = zg(cj, nj);
+            if (__any_sync(0xffffffffu, ei < 600 || ej < 600)) {
+                split_tile<kConjA, false, KS>(g8, zgi, zgj, {ni, nj, zi == zj ? kGram : kFull}, zi == zj, v, ex);
             } else {
                 split_tile_on<kConjA, KS>(
                     g8, [&](int i, int k) { return (FULL || (i < ni && k < m)) ? zi[k * LDZ + i] : zero_on; },
                     [&](int i, int k) { return (FULL || (i < nj && k < m)) ? zj[k * LDZ + i] : zero_on; }, zi == zj, v);
 #pragma unroll
                 for (int j = 0; j < 2; ++j) ex[j] = ei + __shfl_sync(0xffffffffu, ej, 8 * tq + 4 * j);
+                const int *zim = sE + b * SE + 5 * MT;
+                const unsigned im = ((FULL || g < ni) ? zim[ci + g] : 0) | ((FULL || g < nj) ? zim[cj + g] : 0);
+                split_recheck<kConjA, 4>(g8, zgi, zgj, {ni, nj, zi == zj ? kGram : kFull}, im, SplitGrid{ei, ej}, v, ex);
             }
         }
         const int p = 8 * I + g;
@@ -502,17 +509,21 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                 const bool hasL = t >= 1, hasR = 2 * t + 1 < a.Nl;
                 z2 *Zb = sZ + b * MT * LDZ;
                 const z2 *Xb = sL + b * SL;
+                auto xl = [=](int i, int k) { return ((FULL || i < m) && k <= i) ? Xb[tri(i, k)] : zmk(0.0, 0.0); };
                 z2 x[2], z[2][2];
                 SplitCut cx, cz[2];
                 SplitJoint jt[2];
-                unsigned mx[2], mz[2];
+                unsigned mx[2], mz[2], im[2] = {0, 0};
                 bool ok = true;
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
                     const int k = 2 * tq + j;
-                    x[j] = ((FULL || g < m) && k <= g) ? Xb[tri(g, k)] : zero;
+                    x[j] = xl(g, k);
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) z[h][j] = (FULL || (g < m && k < m)) ? Zb[k * LDZ + (h ? m : 0) + g] : zero;
+                    for (int h = 0; h < 2; ++h) {
+                        z[h][j] = (FULL || (g < m && k < m)) ? Zb[k * LDZ + (h ? m : 0) + g] : zero;
+                        im[h] |= im_bits(z[h][j]) | im_bits(x[j]);
+                    }
                     const int64_t o = t * mm + g * m + k;
                     if ((FULL || (g < m && k < m)) && CRS_IN(a, kDbgL, o)) a.L[o] = x[j];
                 }
@@ -528,16 +539,13 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                     SplitAcc acc;
                     split_start(acc, kSplitStart);
                     split_mma<kPlain>(cz[h], cx, acc);
-                    double v[4];
+                    z2 v[2];
+                    split_sums(acc, v);
+                    const z2 *Bs = Zb + (h ? m : 0);
+                    auto bl = [=](int i, int k) { return (FULL || (i < m && k < m)) ? Bs[k * LDZ + i] : zmk(0.0, 0.0); };
+                    if (split_needs<1>(1, bl, xl, {m, m, kFull}, im[h], SplitGridJoint{jt[h].ea}, v)) ok = false;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        int sum[kSplitDigits];
-#pragma unroll
-                        for (int d = 0; d < kSplitDigits; ++d) sum[d] = __float_as_int(acc[d][j]);
-                        v[j] = split_scaled(split_value<1>(sum), jt[h].ea);
-                    }
-                    z[h][0] = zmk(v[0], v[2]);
-                    z[h][1] = zmk(v[1], v[3]);
+                    for (int j = 0; j < 2; ++j) z[h][j] = zmk(split_scaled(v[j].x, jt[h].ea), split_scaled(v[j].y, jt[h].ea));
                     mz[h] = split_max4(max(split_mag(z[h][0]), split_mag(z[h][1])));
                     if (split_unsafe(mz[h])) ok = false;
                 }
@@ -546,7 +554,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                 ok = __all_sync(0xffffffffu, ok);
                 if (lane == 0) sC[b * Split64<MT>::SC].x = ok ? 1.0 : 0.0;
                 __syncwarp();
-                if (!ok) {      // out of the split's range somewhere
+                if (!ok) {      // out of the split's range, or a small entry of Z
                     z_task(b, 0);
                     z_task(b, 1);
                     __syncwarp();
@@ -563,7 +571,10 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                         if ((FULL || (g < m && r < m)) && CRS_IN(a, kDbgZ, o)) a.Z[o] = z[h][j];
                     }
                     split_cut(cz[h], z[h][0], z[h][1], ez[h], ez[h]);
+                    im[h] = im_bits(z[h][0]) | im_bits(z[h][1]);
                 }
+                __syncwarp();       // Z is stored
+                unsigned again = 0;     // products with small entries
                 // P^H P, Q^H P, Q^H Q
 #pragma unroll
                 for (int f = 0; f < 3; ++f) {
@@ -572,21 +583,32 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                     SplitAcc acc;
                     split_start(acc, kSplitStart);
                     split_mma<kConjA>(cz[hi], cz[hj], acc);
+                    z2 v[2];
+                    int ex[2];
+                    split_sums(acc, v);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) ex[j] = ez[hi] + __shfl_sync(0xffffffffu, ez[hj], 8 * tq + 4 * j);
+                    const z2 *Z = a.Z + t * 2 * (int64_t)mm;
+                    auto zl = [=](int h) {
+                        return [=](int i, int k) {
+                            return ((FULL || (i < m && k < m)) && CRS_IN(a, kDbgZ, t * 2 * (int64_t)mm + k * m2 + h * m + i)) ? Z[k * m2 + h * m + i]
+                                                                                                                       : zmk(0.0, 0.0);
+                        };
+                    };
+                    if (split_needs<1>(1, zl(hi), zl(hj), {m, m, f != 1 ? kGram : kFull}, im[hi] | im[hj],
+                                       SplitGrid{ez[hi], ez[hj]}, v)) {
+                        again |= 1u << f;
+                        continue;
+                    }
+                    if (f == 2 && again) continue;      // (Q^H Q takes Z's place in sZ)
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        const int p = g, q = 2 * tq + j, ex = ez[hi] + __shfl_sync(0xffffffffu, ez[hj], 8 * tq + 4 * j);
-                        int s0[kSplitDigits], s1[kSplitDigits];
-#pragma unroll
-                        for (int d = 0; d < kSplitDigits; ++d) {
-                            s0[d] = __float_as_int(acc[d][j]);
-                            s1[d] = __float_as_int(acc[d][j + 2]);
-                        }
-                        const z2 v = zmk(split_value<1>(s0), split_value<1>(s1));
+                        const int p = g, q = 2 * tq + j;
                         if ((!FULL && (p >= m || q >= m)) || (f != 1 && q > p)) continue;
                         if (f == 2) {
-                            Zb[p * LDZ + q] = sub_qq(load_a(b, p, q), p, q, v, ex);
+                            Zb[p * LDZ + q] = sub_qq(load_a(b, p, q), p, q, v[j], ex[j]);
                         } else {
-                            z2 w = zmk(split_scaled(v.x, ex), split_scaled(v.y, ex));
+                            z2 w = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
                             if (f == 1) {
                                 put_qp(b, p, q, w);
                             } else {
@@ -595,6 +617,20 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                             }
                         }
                     }
+                }
+                if (again) {        // by tasks, Q^H Q below
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            const int r = 2 * tq + j;
+                            const int64_t o = t * 2 * (int64_t)mm + r * m2 + (h ? m : 0) + g;
+                            if (FULL || (g < m && r < m)) Zb[r * LDZ + (h ? m : 0) + g] = CRS_IN(a, kDbgZ, o) ? a.Z[o] : zero;
+                        }
+                    if (lane == 0) sC[b * Split64<MT>::SC].x = 0.0;
+                    __syncwarp();
+                    if (again & 1) h_task(b, 0, 0);
+                    if (again & 2) h_task(b, 0, 1);
                 }
             }
             __syncthreads();
@@ -619,10 +655,17 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
         constexpr unsigned kAll = 0xffffffffu;
         for (int e = warp; e < nbh * m; e += nw) {
             const int b = e / m, k = e - b * m;
-            unsigned mx = 0;
-            for (int r = k + lane; r < m; r += 32) mx = max(mx, split_mag(sL[b * SL + tri(r, k)]));
+            unsigned mx = 0, im = 0;
+            for (int r = k + lane; r < m; r += 32) {
+                mx = max(mx, split_mag(sL[b * SL + tri(r, k)]));
+                im |= im_bits(sL[b * SL + tri(r, k)]);
+            }
             for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(kAll, mx, o));
-            if (lane == 0) sE[b * SE + k] = split_unsafe(mx) ? 0 : split_exp(mx);
+            im = __any_sync(kAll, im != 0u);
+            if (lane == 0) {
+                sE[b * SE + k] = split_unsafe(mx) ? 0 : split_exp(mx);
+                sE[b * SE + 4 * MT + k] = im;
+            }
         }
         __syncthreads();
         for (int e = warp; e < nbh * m; e += nw) {
@@ -660,11 +703,13 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
             // B's columns onto the joint grid
             SplitJoint jt;
             bool xbad = false;
+            unsigned im = 0;
             for (int s = 0; s < g8; ++s)
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const int k = 8 * s + 2 * tq + u, c = (FULL || k < m) ? xe[k] : 1023;
                     xbad |= c == 0;
+                    im |= im_bits(zc(k)) | ((FULL || k < m) ? xe[4 * MT + k] : 0);
                     // (a column of X has its diagonal entry)
                     jt.term(split_mag(zc(k)), (unsigned)c << 20);
                 }
@@ -675,6 +720,13 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
             } else if (!ok) {
                 z_task(b, cg);
             } else {
+                const z2 *BL = a.B, *XL = a.L;
+                auto bg = [=](int i, int k) {       // the columns as the level has them
+                    if (!FULL && (i >= nc || k >= m)) return zmk(0.0, 0.0);
+                    const int64_t o = inP ? (2 * t - 1) * mm + k * m + c0 + i : 2 * t * mm + (c0 + i) * m + k;
+                    if (!CRS_IN(a, kDbgB, o)) return zmk(0.0, 0.0);
+                    return inP ? BL[o] : zconj(BL[o]);
+                };
                 for (int s = 0; s < g8; ++s)
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
@@ -684,17 +736,33 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                 __syncwarp();
                 for (int R = g8 - 1; R >= 0; --R) {
                     z2 v[2];
+                    int ex[2];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) ex[j] = jt.ea + ((FULL || 8 * R + 2 * tq + j < m) ? xe[MT + 8 * R + 2 * tq + j] : 0);
                     split_tile_on<kPlain, KS>(
                         R + 1, [&](int i, int k) { return (FULL || (i < nc && k < m)) ? Zb[k * LDZ + col - g + i] : zero_on; },
                         [&](int i, int k) { return ((FULL || 8 * R + i < m) && k <= 8 * R + i) ? Xb[tri(8 * R + i, k)] : zero_on; }, false, v);
+                    auto xg = [=](int i, int k) {
+                        const int64_t o = t * mm + (8 * R + i) * m + k;
+                        return ((FULL || 8 * R + i < m) && k <= 8 * R + i && CRS_IN(a, kDbgL, o)) ? XL[o] : zmk(0.0, 0.0);
+                    };
+                    const int ea = jt.ea, er = (FULL || 8 * R + g < m) ? xe[MT + 8 * R + g] : 0;
+                    auto grid = [=](int s, z2, z2, int (&ga)[2], int (&gb)[2]) {
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const int k = 8 * s + 2 * tq + u, c = (FULL || k < m) ? xe[k] : 1023;
+                            ga[u] = ea - c;
+                            gb[u] = c + er;
+                        }
+                    };
+                    split_recheck<kPlain, 4>(R + 1, bg, xg, {nc, m - 8 * R, kFull}, im, grid, v, ex);
                     __syncwarp();
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const int r = 8 * R + 2 * tq + j;
                         if (FULL || (g < nc && r < m)) {
-                            const int ex = jt.ea + xe[MT + r];
                             const int64_t o = t * m2 * m + r * m2 + col;
-                            const z2 w = zmk(split_scaled(v[j].x, ex), split_scaled(v[j].y, ex));
+                            const z2 w = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
                             Zb[r * LDZ + col] = w;
                             if (CRS_IN(a, kDbgZ, o)) a.Z[o] = w;
                         }
@@ -709,13 +777,22 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                 }
             // Z's columns onto their own grid
             unsigned mx = 0;
+            im = 0;
             for (int s = 0; s < g8; ++s)
 #pragma unroll
-                for (int u = 0; u < 2; ++u) mx = max(mx, split_mag(zc(8 * s + 2 * tq + u)));
+                for (int u = 0; u < 2; ++u) {
+                    const z2 z = zc(8 * s + 2 * tq + u);
+                    mx = max(mx, split_mag(z));
+                    im |= im_bits(z);
+                }
             mx = split_max4(mx);
+            im = split_max4(im);
             const int ez = split_unsafe(mx) ? 0 : split_exp(mx);
             if (FULL || g < nc) {
-                if (tq == 0) ze[col] = ez;
+                if (tq == 0) {
+                    ze[col] = ez;
+                    ze[3 * MT + col] = im != 0u;
+                }
                 for (int s = 0; s < g8; ++s)
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
@@ -767,18 +844,35 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
     const int lane = tid & 31, g = lane >> 2, tq = lane & 3, warp = tid >> 5, nw = NT >> 5;
     const int g8 = (FULL || KS == 1) ? KS : (m + 7) >> 3, ncg = (kw + 7) >> 3, per = g8 * ncg;
 
+    // Operands of block b: columns n0 .. of y_odd, rows 8 R .. of X, columns 8 G ..
+    // of P (h = 0) or Q.
+    auto y_of = [&](int b, int n0) {
+        const int64_t yo = 2 * (t0 + b) * mk + cb + n0;
+        const z2 *y = a.y;
+        const int nc = kw - n0;
+        return [=](int i, int s) { return (i < nc && (FULL || s < m) && CRS_IN(a, kDbgY, yo + s * k + i)) ? y[yo + s * k + i] : zmk(0.0, 0.0); };
+    };
+    auto x_of = [&](int b, int R) {
+        const int64_t xo = (t0 + b) * mm + 8 * R * m;
+        const z2 *X = a.L;
+        return [=](int i, int s) {
+            return ((FULL || 8 * R + i < m) && s <= 8 * R + i && CRS_IN(a, kDbgL, xo + i * m + s)) ? X[xo + i * m + s] : zmk(0.0, 0.0);
+        };
+    };
+    auto z_of = [&](int b, int h, int G) {
+        const int64_t zo = (t0 + b) * m2 * m + (h ? m : 0) + 8 * G;
+        const z2 *Z = a.Z;
+        return [=](int i, int s) {
+            return ((FULL || (8 * G + i < m && s < m)) && CRS_IN(a, kDbgZ, zo + s * m2 + i)) ? Z[zo + s * m2 + i] : zmk(0.0, 0.0);
+        };
+    };
     // r of rows 8 R .. and columns n0 .. of block b
     auto r_task = [&](int b, int R, int n0) {
-        const int64_t t = t0 + b, yo = 2 * t * mk + cb + n0, xo = t * mm + 8 * R * m;
+        const int64_t t = t0 + b;
         const int nc = kw - n0;
         z2 v[2];
         int ex[2];
-        split_tile<kPlain, true, KS>(
-            R + 1, [&](int i, int s) { return (i < nc && (FULL || s < m) && CRS_IN(a, kDbgY, yo + s * k + i)) ? a.y[yo + s * k + i] : zero; },
-            [&](int i, int s) {
-                return ((FULL || 8 * R + i < m) && s <= 8 * R + i && CRS_IN(a, kDbgL, xo + i * m + s)) ? a.L[xo + i * m + s] : zero;
-            },
-            false, v, ex);
+        split_tile<kPlain, true, KS>(R + 1, y_of(b, n0), x_of(b, R), {nc, m - 8 * R, kFull}, false, v, ex);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int r = 8 * R + 2 * tq + j;
@@ -815,7 +909,7 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
     // rows 8 G .. of P^H r (pass 0) or Q^H r (pass 1); keep: y_even - Q^H r goes to
     // sR in the place of r
     auto u_task = [&](int b, int pass, int G, int n0, bool keep) {
-            const int64_t t = t0 + b, zo = t * m2 * m + (pass ? m : 0) + 8 * G;
+            const int64_t t = t0 + b;
             if (pass ? 2 * t + 1 >= a.Nl : t < 1) return;
             const int nc = kw - n0, np = m - 8 * G;
             const z2 *Rb = sR + b * MT * kc + n0;
@@ -824,9 +918,8 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
 #pragma unroll
             for (int j = 0; j < 2; ++j) u[j] = pass ? load_y(b, 8 * G + g, n0 + 2 * tq + j) : zero;
             split_tile<kConjA, false, KS>(
-                g8,
-                [&](int i, int s) { return ((FULL || (i < np && s < m)) && CRS_IN(a, kDbgZ, zo + s * m2 + i)) ? a.Z[zo + s * m2 + i] : zero; },
-                [&](int i, int s) { return (i < nc && (FULL || s < m)) ? Rb[s * kc + i] : zero; }, false, v, ex);
+                g8, z_of(b, pass, G),
+                [=](int i, int s) { return (i < nc && (FULL || s < m)) ? Rb[s * kc + i] : zmk(0.0, 0.0); }, {np, nc, kFull}, false, v, ex);
             if (keep) __syncwarp();     // sR is read up to here
             const int p = 8 * G + g;
 #pragma unroll
@@ -865,6 +958,7 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
                 u[j] = load_y(b, g, n0 + s);
             }
             unsigned mx[2], mz[2];
+            unsigned im = im_bits(y[0]) | im_bits(y[1]) | im_bits(x[0]) | im_bits(x[1]);
             SplitJoint jt;
             split_joint_exp(x[0], x[1], mx[0], mx[1]);
             jt.term(split_mag(y[0]), mx[0]);
@@ -883,21 +977,15 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
                 split_cut(c2, x[0], x[1], e0, e1);
                 split_start(acc, kSplitStart);
                 split_mma<kPlain>(c1, c2, acc);
-            }
+                split_sums(acc, r);
+                if (split_needs<1>(1, y_of(b, n0), x_of(b, 0), {nc, m, kFull}, im, SplitGridJoint{jt.ea}, r)) ok = false;
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                int s0[kSplitDigits], s1[kSplitDigits];
-#pragma unroll
-                for (int d = 0; d < kSplitDigits; ++d) {
-                    s0[d] = __float_as_int(acc[d][j]);
-                    s1[d] = __float_as_int(acc[d][j + 2]);
-                }
-                r[j] = zmk(split_scaled(split_value<1>(s0), jt.ea), split_scaled(split_value<1>(s1), jt.ea));
+                for (int j = 0; j < 2; ++j) r[j] = zmk(split_scaled(r[j].x, jt.ea), split_scaled(r[j].y, jt.ea));
             }
             const unsigned mr = split_max4(max(split_mag(r[0]), split_mag(r[1])));
             const int er = split_exp(mr);
             if (split_unsafe(mr) || er < kSplitSumTiny / 2) ok = false;
-            if (!__all_sync(kAll, ok)) {        // out of the split's range somewhere
+            if (!__all_sync(kAll, ok)) {        // out of the split's range, or a small entry of r
                 r_task(b, 0, n0);
                 __syncwarp();
                 u_task(b, 0, 0, n0, false);
@@ -911,6 +999,9 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
                 if (g < nc && (FULL || 2 * tq + j < m) && CRS_IN(a, kDbgR, o)) a.r[o] = r[j];
             }
             split_cut(c2, r[0], r[1], er, er);
+            const unsigned ir = im_bits(r[0]) | im_bits(r[1]);
+            __syncwarp();       // r is stored
+            unsigned again = 0;     // products with small entries
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 if (h ? !hasR : !hasL) continue;
@@ -918,24 +1009,40 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
                 split_cut(c1, z[h][0], z[h][1], ez, ez);
                 split_start(acc, kSplitStart);
                 split_mma<kConjA>(c1, c2, acc);
+                z2 v[2];
+                int ex[2];
+                split_sums(acc, v);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) ex[j] = ez + __shfl_sync(kAll, er, 8 * tq + 4 * j);
+                const int64_t ro = t * mk + cb + n0;
+                const z2 *Rg = a.r;
+                auto rl = [=](int i, int s) {
+                    return (i < nc && (FULL || s < m) && CRS_IN(a, kDbgR, ro + s * k + i)) ? Rg[ro + s * k + i] : zmk(0.0, 0.0);
+                };
+                if (split_needs<1>(1, z_of(b, h, 0), rl, {m, nc, kFull}, ir | im_bits(z[h][0]) | im_bits(z[h][1]),
+                                   SplitGrid{ez, er}, v)) {
+                    again |= 1u << h;
+                    continue;
+                }
+                if (h == 1 && again) continue;      // (y - Q^H r takes the place of r in sR)
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    const int ex = ez + __shfl_sync(kAll, er, 8 * tq + 4 * j), n = 2 * tq + j;
-                    int s0[kSplitDigits], s1[kSplitDigits];
-#pragma unroll
-                    for (int d = 0; d < kSplitDigits; ++d) {
-                        s0[d] = __float_as_int(acc[d][j]);
-                        s1[d] = __float_as_int(acc[d][j + 2]);
-                    }
-                    const z2 v = zmk(split_value<1>(s0), split_value<1>(s1));
+                    const int n = 2 * tq + j;
                     if ((!FULL && g >= m) || n >= nc) continue;
                     if (h == 0) {
-                        put_pr(b, g, n0 + n, zmk(split_scaled(v.x, ex), split_scaled(v.y, ex)));
+                        put_pr(b, g, n0 + n, zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j])));
                     } else {
-                        const double sc = -split_scale(ex);
-                        sR[(b * MT + g) * kc + n0 + n] = zmk(fma(v.x, sc, u[j].x), fma(v.y, sc, u[j].y));
+                        const double sc = -split_scale(ex[j]);
+                        sR[(b * MT + g) * kc + n0 + n] = zmk(fma(v[j].x, sc, u[j].x), fma(v[j].y, sc, u[j].y));
                     }
                 }
+            }
+            if (again) {        // by tasks
+                r_task(b, 0, n0);
+                __syncwarp();
+                if (again & 1) u_task(b, 0, 0, n0, false);
+                __syncwarp();
+                u_task(b, 1, 0, n0, true);
             }
         }
         __syncthreads();
@@ -1002,10 +1109,42 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
     }
     if (failed) return;
 
-    auto w_task = [&](int b, int R, int n0) {
-        const int64_t t = t0 + b, zo = t * m2 * m + 8 * R * m2;
-        const int nc = kw - n0;
+    // Operands of block b: columns n0 .. of [x_left; x_right] and rows 8 R .. of [P | Q]
+    // (terms 0 .. 8 g8 - 1: P and x_left, 8 g8 .. : Q and x_right), columns 8 G .. of
+    // X from row 8 G on (X[s][p] is zero for s < p).
+    auto xn_of = [&](int b, int n0) {
+        const int64_t t = t0 + b, xo = t * mk + cb + n0;
         const bool hasL = t >= 1, hasR = t < a.ne;
+        const z2 *xn = a.xn;
+        const int nc = kw - n0;
+        return [=](int i, int s) {
+            const bool right = s >= 8 * g8;
+            const int q = right ? s - 8 * g8 : s;
+            const int64_t o = xo + (right ? 0 : -mk) + q * k + i;
+            return (i < nc && (FULL || q < m) && (right ? hasR : hasL) && CRS_IN(a, kDbgXn, o)) ? xn[o] : zmk(0.0, 0.0);
+        };
+    };
+    auto z_of = [&](int b, int R) {
+        const int64_t zo = (t0 + b) * m2 * m + 8 * R * m2;
+        const z2 *Z = a.Z;
+        return [=](int i, int s) {
+            const bool right = s >= 8 * g8;
+            const int q = right ? s - 8 * g8 : s;
+            const int64_t o = zo + i * m2 + (right ? m : 0) + q;
+            return ((FULL || (8 * R + i < m && q < m)) && CRS_IN(a, kDbgZ, o)) ? Z[o] : zmk(0.0, 0.0);
+        };
+    };
+    auto x_of = [&](int b, int G) {
+        const int64_t xo = (t0 + b) * mm + 8 * G * m + 8 * G;
+        const int np = m - 8 * G;
+        const z2 *X = a.L;
+        return [=](int i, int s) {
+            return ((FULL || (i < np && s < np)) && i <= s && CRS_IN(a, kDbgL, xo + s * m + i)) ? X[xo + s * m + i] : zmk(0.0, 0.0);
+        };
+    };
+    auto w_task = [&](int b, int R, int n0) {
+        const int64_t t = t0 + b;
+        const int nc = kw - n0;
         z2 v[2], u[2];
         int ex[2];
 #pragma unroll
@@ -1013,22 +1152,7 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
             const int64_t o = t * mk + (int64_t)(8 * R + 2 * tq + j) * k + cb + n0 + g;
             u[j] = (g < nc && (FULL || 8 * R + 2 * tq + j < m) && CRS_IN(a, kDbgR, o)) ? a.r[o] : zero;
         }
-        // terms 0 .. 8 g8 - 1: P and x_left, 8 g8 .. : Q and x_right
-        split_tile<kPlain, true, 2 * KS>(
-            2 * g8,
-            [&](int i, int s) {
-                const bool right = s >= 8 * g8;
-                const int q = right ? s - 8 * g8 : s;
-                const int64_t o = (right ? t : t - 1) * mk + q * k + cb + n0 + i;
-                return (i < nc && (FULL || q < m) && (right ? hasR : hasL) && CRS_IN(a, kDbgXn, o)) ? a.xn[o] : zero;
-            },
-            [&](int i, int s) {
-                const bool right = s >= 8 * g8;
-                const int q = right ? s - 8 * g8 : s;
-                const int64_t o = zo + i * m2 + (right ? m : 0) + q;
-                return ((FULL || (8 * R + i < m && q < m)) && CRS_IN(a, kDbgZ, o)) ? a.Z[o] : zero;
-            },
-            false, v, ex);
+        split_tile<kPlain, true, 2 * KS>(2 * g8, xn_of(b, n0), z_of(b, R), {nc, m - 8 * R, kFull}, false, v, ex);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int r = 8 * R + 2 * tq + j;
@@ -1041,15 +1165,14 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
         }
     };
     auto x_task = [&](int b, int G, int n0) {
-        const int64_t t = t0 + b, xo = t * mm + 8 * G * m + 8 * G;
+        const int64_t t = t0 + b;
         const int nc = kw - n0, np = m - 8 * G;
         const z2 *Wb = sW + (b * MT + 8 * G) * kc + n0;
         z2 v[2];
         int ex[2];
-        // X[s][p] is zero for s < p: terms from row 8 G on
         split_tile<kConjA, false, KS>(
-            g8 - G, [&](int i, int s) { return ((FULL || (i < np && s < np)) && i <= s && CRS_IN(a, kDbgL, xo + s * m + i)) ? a.L[xo + s * m + i] : zero; },
-            [&](int i, int s) { return (i < nc && (FULL || s < np)) ? Wb[s * kc + i] : zero; }, false, v, ex);
+            g8 - G, x_of(b, G),
+            [=](int i, int s) { return (i < nc && (FULL || s < np)) ? Wb[s * kc + i] : zmk(0.0, 0.0); }, {np, nc, kFull}, false, v, ex);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int p = 8 * G + g, n = 2 * tq + j;
@@ -1082,13 +1205,14 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
                 const int64_t oe = (2 * t + 1) * mk + (int64_t)s * k + cb + n0 + g;
                 if (col && t < a.ne && CRS_IN(a, kDbgX, oe)) a.x[oe] = xn[1][j];
             }
-            unsigned mx[2][2];
+            unsigned mx[2][2], im = 0;
             SplitJoint jt;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 split_joint_exp(z[h][0], z[h][1], mx[h][0], mx[h][1]);
                 jt.term(split_mag(xn[h][0]), mx[h][0]);
                 jt.term(split_mag(xn[h][1]), mx[h][1]);
+                im |= im_bits(z[h][0]) | im_bits(z[h][1]) | im_bits(xn[h][0]) | im_bits(xn[h][1]);
             }
             bool ok = !jt.finish() && jt.ea >= kSplitSumTiny;
             const unsigned ml = split_max4(max(split_mag(x[0]), split_mag(x[1])));
@@ -1103,22 +1227,31 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
                 split_cut(c2, z[h][0], z[h][1], e0, e1);
                 split_mma<kPlain>(c1, c2, acc);
             }
-            const double sc = -split_scale(jt.ea);
+            {
+                z2 v[2];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                int s0[kSplitDigits], s1[kSplitDigits];
+                for (int j = 0; j < 2; ++j) {
+                    int s0[kSplitDigits], s1[kSplitDigits];
 #pragma unroll
-                for (int d = 0; d < kSplitDigits; ++d) {
-                    s0[d] = __float2int_rn(acc[d][j]);
-                    s1[d] = __float2int_rn(acc[d][j + 2]);
+                    for (int d = 0; d < kSplitDigits; ++d) {
+                        s0[d] = __float2int_rn(acc[d][j]);
+                        s1[d] = __float2int_rn(acc[d][j + 2]);
+                    }
+                    v[j] = zmk(split_value<2>(s0), split_value<2>(s1));
                 }
-                w[j].x = fma(split_value<2>(s0), sc, w[j].x);
-                w[j].y = fma(split_value<2>(s1), sc, w[j].y);
+                if (split_needs<2>(2, xn_of(b, n0), z_of(b, 0), {nc, m, kFull}, im, SplitGridJoint{jt.ea}, v)) ok = false;
+                const double sc = -split_scale(jt.ea);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    w[j].x = fma(v[j].x, sc, w[j].x);
+                    w[j].y = fma(v[j].y, sc, w[j].y);
+                }
             }
             const unsigned mw = split_max4(max(split_mag(w[0]), split_mag(w[1])));
             const int ew = split_exp(mw), el = split_exp(ml);
             if (split_unsafe(mw) || ew < kSplitSumTiny / 2) ok = false;
-            if (!__all_sync(kAll, ok)) {        // out of the split's range somewhere
+            // by tasks: out of the split's range, or a small entry
+            if (!__all_sync(kAll, ok)) {
                 w_task(b, 0, n0);
                 __syncwarp();
                 x_task(b, 0, n0);
@@ -1128,18 +1261,30 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
             split_cut(c2, w[0], w[1], ew, ew);
             split_start(acc, kSplitStart);
             split_mma<kConjA>(c1, c2, acc);
+            z2 v[2];
+            int ex[2];
+            split_sums(acc, v);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) ex[j] = el + __shfl_sync(kAll, ew, 8 * tq + 4 * j);
+            const z2 *Wb = sW + b * MT * kc + n0;
+            auto wl = [=](int i, int s) {       // (of the block, put into sW for this look)
+                return (i < nc && (FULL || s < m)) ? Wb[s * kc + i] : zmk(0.0, 0.0);
+            };
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                if (g < nc && (FULL || 2 * tq + j < m)) sW[(b * MT + 2 * tq + j) * kc + n0 + g] = w[j];
+            __syncwarp();
+            if (split_needs<1>(1, x_of(b, 0), wl, {m, nc, kFull}, im_bits(x[0]) | im_bits(x[1]) | im_bits(w[0]) | im_bits(w[1]),
+                               SplitGrid{el, ew}, v)) {
+                x_task(b, 0, n0);
+                continue;
+            }
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-                const int ex = el + __shfl_sync(kAll, ew, 8 * tq + 4 * j), n = 2 * tq + j;
-                int s0[kSplitDigits], s1[kSplitDigits];
-#pragma unroll
-                for (int d = 0; d < kSplitDigits; ++d) {
-                    s0[d] = __float_as_int(acc[d][j]);
-                    s1[d] = __float_as_int(acc[d][j + 2]);
-                }
+                const int n = 2 * tq + j;
                 const int64_t o = 2 * t * mk + (int64_t)g * k + cb + n0 + n;
                 if ((FULL || g < m) && n < nc && CRS_IN(a, kDbgX, o))
-                    a.x[o] = zmk(split_scaled(split_value<1>(s0), ex), split_scaled(split_value<1>(s1), ex));
+                    a.x[o] = zmk(split_scaled(v[j].x, ex[j]), split_scaled(v[j].y, ex[j]));
             }
         }
     } else {

@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(256) k_solve_up_wide(LevelArgsT<R> a) {
 // The split forms of the FP64 levels (cr_core64.cuh).
 // (class 64 at twice the tile's threads: split_threads)
 template <int MT>
-__global__ void __launch_bounds__(MT == 64 ? 512 : 256) k_factor_split(LevelArgs a) {
+__global__ void __launch_bounds__(MT == 64 ? 512 : 256, MT == 8 ? 2 : 0) k_factor_split(LevelArgs a) {
     level_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     factor_chunk_split<MT>(a, a.c_begin + blockIdx.x, smem_raw);
@@ -158,7 +158,6 @@ __global__ void __launch_bounds__(256) k_adjoint_outer_split(int64_t N, int m, i
     const int g8 = (m + 7) >> 3, ntri = g8 * (g8 + 1) / 2, nA = gA ? ntri : 0, per = nA + (gB ? g8 * g8 : 0);
     const int lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
     const int64_t mk = (int64_t)m * k, mm = (int64_t)m * m, nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const z2 zero = zmk(0.0, 0.0);
     for (int64_t e = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); e < N * per; e += nw) {
         const int64_t j = e / per;
         const int f = (int)(e - j * per);
@@ -178,15 +177,15 @@ __global__ void __launch_bounds__(256) k_adjoint_outer_split(int64_t N, int m, i
         int ex[2];
         split_tile<kConjB, true, KS>(
             (2 * k + 7) >> 3,
-            [&](int i, int s) {
+            [=](int i, int s) {
                 const bool h = s >= k;
-                return (i < ni && s < 2 * k) ? __ldg((h ? x : gy) + o1 + i * k + (h ? s - k : s)) : zero;
+                return (i < ni && s < 2 * k) ? __ldg((h ? x : gy) + o1 + i * k + (h ? s - k : s)) : zmk(0.0, 0.0);
             },
-            [&](int i, int s) {
+            [=](int i, int s) {
                 const bool h = s >= k;
-                return (i < nj && s < 2 * k) ? __ldg((h ? gy : x) + o0 + i * k + (h ? s - k : s)) : zero;
+                return (i < nj && s < 2 * k) ? __ldg((h ? gy : x) + o0 + i * k + (h ? s - k : s)) : zmk(0.0, 0.0);
             },
-            false, v, ex);
+            {ni, nj, isA && I == J ? kHermitian : kFull}, false, v, ex);
         const int p = 8 * I + g;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {

@@ -21,6 +21,13 @@
 // rounded once.  The error is thus that of one rounding of the result plus
 // about 2^-56 max|a| max|b| sqrt(K), where a chain of FP64 FMAs rounds K times.
 //
+// That second part is measured by the largest entries.  A result whose own terms
+// are all much smaller (a localised source, rows of other units, a tiny imaginary
+// part) would keep few or none of its bits, where FMAs keep them all.  Such
+// results are told by their size and by their operands, and formed by FMAs
+// (split_guard), so that every result is good to a few ulp of the sum of its
+// own terms' magnitudes.
+//
 // Cutting is integer work and bounds these kernels (the integer pipe does 64
 // lanes per clock per SM, measured): digits of a byte need no shifts, only a
 // byte permute and a mask for two entries, which is why there are seven of
@@ -197,6 +204,20 @@ __host__ __device__ __forceinline__ double split_value(const int (&s)[kSplitDigi
     return (double)(int64_t)v;
 }
 
+// The lane's two entries of a tile of one K-step.
+__device__ __forceinline__ void split_sums(const SplitAcc &acc, z2 (&v)[2]) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        int s0[kSplitDigits], s1[kSplitDigits];
+#pragma unroll
+        for (int d = 0; d < kSplitDigits; ++d) {
+            s0[d] = __float_as_int(acc[d][j]);
+            s1[d] = __float_as_int(acc[d][j + 2]);
+        }
+        v[j] = zmk(split_value<1>(s0), split_value<1>(s1));
+    }
+}
+
 // v times 2^(k - 2100) for a value of split_value and a sum k of two biased
 // exponents, by the exponent field (no FP64 instruction); and that factor.
 __device__ __forceinline__ double split_scaled(double v, int k) {
@@ -209,7 +230,7 @@ __device__ __forceinline__ double split_scale(int k) { return __hiloint2double((
 // by one warp: lane (g, t) = (lane / 4, lane % 4) gets the entries
 // (row g, columns 2t + j), j = 0, 1, as v[j] times 2^(e[j] - 2100).
 // la(i, k): entry k of row i of the first operand, lb(i, k): entry k of column
-// i of the second; both return zero outside the block.
+// i of the second; both return zero outside the block, and capture by value.
 //
 // Scaling.  kJoint = false: rows of the first and columns of the second
 // operand each on their own binary grid.  kJoint = true, for products X b
@@ -219,8 +240,9 @@ __device__ __forceinline__ double split_scale(int k) { return __hiloint2double((
 // scaling of the unknowns (X_ik -> X_ik / d_k, b_k -> d_k b_k) leaves such a
 // product's digits as they are, as it leaves the rounding errors of FP64 FMAs.
 //
-// Entries whose row or column leaves the split's range are formed by FP64 FMAs
-// (e[j] = 2100).
+// Entries whose row or column leaves the split's range, and those that
+// split_guard tells, are formed by FP64 FMAs (e[j] = 2100).  use(i, c): which
+// parts of entry (i, c) the caller uses (SplitUse).
 //
 // same: both operands are the same columns (cut once).
 __device__ __forceinline__ unsigned split_mag(z2 z) { return max(mag_hi(z.x), mag_hi(z.y)); }
@@ -270,8 +292,241 @@ __device__ __forceinline__ unsigned split_max4(unsigned m) {
     return max(m, __shfl_xor_sync(0xffffffffu, m, 2));
 }
 
+// ---- results much smaller than their grids' product g = 2^(Ea + Eb)
+//
+// The error of a result over K real terms is below K 2^-53.3 g (two operands off by
+// less than 2^-56 of their grids, dropped digits below 2^-55.3 g, per term).  A
+// result is kept where that is small against the sum S of its own terms' magnitudes:
+// where its modulus is at least 2^-8 g and the part (real or imaginary) at least
+// 2^-14 g, or where one of its real products is at least 2^-8 g.  Its error is then
+// below K 2^-45.3 times the moduli's sum and K 2^-39.3 S, in the worst case that the
+// largest errors of all terms add up (they have either sign).  Else, if any product is
+// not zero, the entry is formed by FMAs.  On the random systems 1% of the
+// tiles come here for a look at their operands, most of them (single-term rows of
+// triangles) also for the FMAs; where entries decay inside a block, most tiles do.
+constexpr int kSplitMod = 8, kSplitPart = 14, kSplitBig = 4;
+
+__device__ __forceinline__ bool nonzero(double v) {
+    return ((unsigned)__double2hiint(v) << 1 | (unsigned)__double2loint(v)) != 0u;
+}
+__device__ __forceinline__ bool nonzero(z2 z) { return nonzero(z.x) || nonzero(z.y); }
+
+// Bits 0 and 1: the real and the imaginary part of a tile's result (in units of
+// split_value<KS>) may have lost bits.
+template <int KS>
+__device__ __forceinline__ unsigned split_small(z2 v) {
+    constexpr unsigned one = 1023 + (KS > 8 ? 53 : 54), mod = (one - kSplitMod) << 20, part = (one - kSplitPart) << 20;
+    const unsigned x = mag_hi(v.x), y = mag_hi(v.y);
+    return max(x, y) < mod ? 3u : (x < part ? 1u : 0u) | (y < part ? 2u : 0u);
+}
+
+// The parts of a tile's entries that a caller uses and that can be small (bits as
+// of split_small): rows i < na and columns c < nb.  kHermitian: of a Hermitian tile
+// the lower triangle, the diagonal real; kGram: without the diagonal, a sum of
+// squares of at least g.
+enum SplitShape { kFull, kHermitian, kGram };
+struct SplitUse {
+    int na, nb;
+    SplitShape shape;
+    __device__ __forceinline__ unsigned operator()(int i, int c) const {
+        if (i >= na || c >= nb) return 0u;
+        if (shape == kFull || c < i) return 3u;
+        return shape == kHermitian && c == i ? 1u : 0u;
+    }
+};
+
+// Which results of a lane have a product that is not zero (nz), or one of at
+// least 2^-8 g (big): bits 2 j + (0: real, 1: imaginary part) of entry (g, 2t + j).
+struct SplitSeen {
+    unsigned nz = 0, big = 0;
+    // one of the lane's terms: a of row g, b of column g, with their grids' exponents
+    __device__ __forceinline__ void term(z2 a, int ea, z2 b, int eb) {
+        constexpr unsigned kAll = 0xffffffffu;
+        const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+        auto near = [](double v, int e) { return (int)(mag_hi(v) >> 20) >= e - kSplitBig; };
+        const unsigned n[4] = {__ballot_sync(kAll, nonzero(a.x)), __ballot_sync(kAll, nonzero(a.y)), __ballot_sync(kAll, nonzero(b.x)),
+                               __ballot_sync(kAll, nonzero(b.y))};
+        const unsigned l[4] = {__ballot_sync(kAll, near(a.x, ea)), __ballot_sync(kAll, near(a.y, ea)),
+                               __ballot_sync(kAll, near(b.x, eb)), __ballot_sync(kAll, near(b.y, eb))};
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            // the four lanes of row g and those of column 2t + j
+            const int r = 4 * g, c = 4 * (2 * t + j);
+            auto parts = [&](const unsigned (&v)[4]) {
+                const unsigned ar = v[0] >> r, ai = v[1] >> r, br = v[2] >> c, bi = v[3] >> c;
+                return ((((ar & br) | (ai & bi)) & 15u) != 0u ? 1u : 0u) | ((((ar & bi) | (ai & br)) & 15u) != 0u ? 2u : 0u);
+            };
+            nz |= parts(n) << (2 * j);
+            big |= parts(l) << (2 * j);
+        }
+    }
+};
+
+// A lane's entries (g, 2t + j) with fma[j] by FMAs over n terms (n a multiple of 8).
+// The warp goes through the terms together, without a branch on fma.
+template <SplitKind KIND, class LA, class LB>
+__device__ __forceinline__ void split_entries(int n, LA la, LB lb, const bool (&fma)[2], z2 (&v)[2], int (&ex)[2]) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, c = 2 * (lane & 3);
+    if (!__any_sync(0xffffffffu, fma[0] | fma[1])) return;
+    z2 r[2] = {zmk(0.0, 0.0), zmk(0.0, 0.0)};
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) {
+        const z2 x = la(g, k);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const z2 y = lb(c + j, k);
+            if constexpr (KIND == kConjA) zmac_ca(r[j], x, y);
+            else if constexpr (KIND == kPlain) zmac(r[j], x, y);
+            else zmac_cb(r[j], x, y);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        v[j].x = fma[j] ? r[j].x : v[j].x;
+        v[j].y = fma[j] ? r[j].y : v[j].y;
+        ex[j] = fma[j] ? 2100 : ex[j];
+    }
+}
+
+// Grids of a product for split_guard: the exponents of a lane's two terms of K-step s.
+struct SplitGrid {          // rows and columns on their own
+    int ea, eb;
+    __device__ __forceinline__ void operator()(int, z2, z2, int (&ga)[2], int (&gb)[2]) const {
+        ga[0] = ga[1] = ea;
+        gb[0] = gb[1] = eb;
+    }
+};
+struct SplitGridJoint {     // rows of exponent sum ea on the terms' own
+    int ea;
+    __device__ __forceinline__ void operator()(int, z2 b0, z2 b1, int (&ga)[2], int (&gb)[2]) const {
+        unsigned m0, m1;
+        split_joint_exp(b0, b1, m0, m1);
+        ga[0] = ea - (gb[0] = split_exp(m0));
+        ga[1] = ea - (gb[1] = split_exp(m1));
+    }
+};
+
+// Which of a lane's entries with small parts (bits of split_small) to form by FMAs.
+// For all lanes of a warp.
+template <class LA, class LB, class GRID>
+__device__ __forceinline__ void split_guard(int ks, LA la, LB lb, GRID grid, const unsigned (&small)[2], bool (&need)[2]) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    SplitSeen seen;
+#pragma unroll 1
+    for (int s = 0; s < ks; ++s) {
+        z2 a[2], b[2];
+        int ea[2], eb[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            a[u] = la(g, 8 * s + 2 * t + u);
+            b[u] = lb(g, 8 * s + 2 * t + u);
+        }
+        grid(s, b[0], b[1], ea, eb);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) seen.term(a[u], ea[u], b[u], eb[u]);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) need[j] = (small[j] & ((seen.nz & ~seen.big) >> (2 * j))) != 0u;
+}
+
+// The imaginary part of an operand as bits, 0: none.
+__device__ __forceinline__ unsigned im_bits(z2 z) { return (unsigned)__double2hiint(z.y) << 1; }
+
+// Are the warp's operands, of whose bits im is the OR, all real?
+__device__ __forceinline__ bool split_real(unsigned im) { return !__any_sync(0xffffffffu, im != 0u); }
+
+// Has any lane a result that split_small tells of, among those that the caller uses?
+template <int KS>
+__device__ __forceinline__ bool split_any_small(SplitUse use, bool real, const z2 (&v)[2]) {
+    constexpr unsigned one = 1023 + (KS > 8 ? 53 : 54), mod = (one - kSplitMod) << 20, part = (one - kSplitPart) << 20;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    bool any = false;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const unsigned x = mag_hi(v[j].x), y = mag_hi(v[j].y);
+        const unsigned p = use(g, 2 * t + j);
+        any |= (max(x, y) < mod || min(x, real || p == 1u ? x : y) < part) && p != 0u;
+    }
+    return any;
+}
+
+// small[j]: the parts of the lane's result v[j] that may have lost bits.
+template <int KS>
+__device__ __forceinline__ bool split_smalls(SplitUse use, bool real, const z2 (&v)[2], unsigned (&small)[2]) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) small[j] = split_small<KS>(v[j]) & use(g, 2 * t + j) & (real ? 1u : 3u);
+    return __any_sync(0xffffffffu, (small[0] | small[1]) != 0u);
+}
+
+// The uncommon cases of a product, out of line so that they cost the kernels no
+// registers: la, lb and grid are taken by value and capture no references.  They
+// are called by whole warps and end converged, as the callers go on to warp-wide
+// instructions.
+
+// Has a product with small results one to form by FMAs in any lane?
+template <int KS, class LA, class LB, class GRID>
+__device__ __noinline__ bool split_look(int ks, LA la, LB lb, GRID grid, SplitUse use, bool real, z2 v0, z2 v1) {
+    const z2 v[2] = {v0, v1};
+    unsigned small[2];
+    if (!split_smalls<KS>(use, real, v, small)) return false;
+    bool need[2];
+    split_guard(ks, la, lb, grid, small, need);
+    return __any_sync(0xffffffffu, need[0] | need[1]);
+}
+
+// Results v, e of a tile after its entries with bad[j], small results that need it
+// and exponents below the normal range.
+struct SplitOut {
+    z2 v[2];
+    int e[2];
+};
+template <SplitKind KIND, int KS, class LA, class LB, class GRID>
+__device__ __noinline__ SplitOut split_slow(int ks, LA la, LB lb, GRID grid, SplitUse use, bool real, bool bad0, bool bad1, SplitOut o) {
+    const bool bad[2] = {bad0, bad1};
+    bool need[2] = {false, false};
+    unsigned small[2];
+    if (split_smalls<KS>(use, real, o.v, small)) split_guard(ks, la, lb, grid, small, need);
+    // each entry decides for itself, so that it does not depend on which
+    // columns share its tile
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        need[j] = need[j] || bad[j];
+        if (!need[j] && o.e[j] < kSplitSumTiny) {
+            // two exact factors down to the last, which rounds into the subnormal range
+            const double s0 = split_scale(2100 - 950), s1 = split_scale(o.e[j] + 950);
+            o.v[j].x = o.v[j].x * s0 * s1;
+            o.v[j].y = o.v[j].y * s0 * s1;
+            o.e[j] = 2100;
+        }
+    }
+    split_entries<KIND>(8 * ks, la, lb, need, o.v, o.e);
+    __syncwarp();
+    return o;
+}
+
+// split_look for results v of operands in the split's range.
+template <int KS, class LA, class LB, class GRID>
+__device__ __forceinline__ bool split_needs(int ks, LA la, LB lb, SplitUse use, unsigned im, GRID grid, const z2 (&v)[2]) {
+    const bool real = split_real(im);
+    return __any_sync(0xffffffffu, split_any_small<KS>(use, real, v)) && split_look<KS>(ks, la, lb, grid, use, real, v[0], v[1]);
+}
+// ... with the FMAs.
+template <SplitKind KIND, int KS, class LA, class LB, class GRID>
+__device__ __forceinline__ void split_recheck(int ks, LA la, LB lb, SplitUse use, unsigned im, GRID grid, z2 (&v)[2], int (&ex)[2]) {
+    const bool real = split_real(im);
+    if (!__any_sync(0xffffffffu, split_any_small<KS>(use, real, v))) return;
+    const SplitOut o = split_slow<KIND, KS>(ks, la, lb, grid, use, real, false, false, SplitOut{{v[0], v[1]}, {ex[0], ex[1]}});
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        v[j] = o.v[j];
+        ex[j] = o.e[j];
+    }
+}
+
 template <SplitKind KIND, bool kJoint, int KS, class LA, class LB>
-__device__ __forceinline__ void split_tile(int ks, LA la, LB lb, bool same, z2 (&v)[2], int (&e)[2]) {
+__device__ __forceinline__ void split_tile(int ks, LA la, LB lb, SplitUse use, bool same, z2 (&v)[2], int (&e)[2]) {
     constexpr unsigned kAll = 0xffffffffu;
     // up to two K-steps the lane keeps its operands in registers between the
     // pass for the exponents and the products; beyond, it loads them again
@@ -298,8 +553,9 @@ __device__ __forceinline__ void split_tile(int ks, LA la, LB lb, bool same, z2 (
         }
     }
     SplitJoint jt;
-    unsigned ma = 0, mb = 0;
+    unsigned ma = 0, mb = 0, im = 0;
     auto exps = [&](int i) {
+        im |= im_bits(a[i][0]) | im_bits(a[i][1]) | im_bits(b[i][0]) | im_bits(b[i][1]);
         if constexpr (kJoint) {
             split_joint_exp(b[i][0], b[i][1], m0[i], m1[i]);
             jt.term(split_mag(a[i][0]), m0[i]);
@@ -387,35 +643,28 @@ __device__ __forceinline__ void split_tile(int ks, LA la, LB lb, bool same, z2 (
         v[j] = zmk(split_value<KS>(sum[j]), split_value<KS>(sum[j + 2]));
         e[j] = ea + (kJoint ? 0 : __shfl_sync(kAll, eb, 8 * t + 4 * j)) + (KS > 8 ? 1 : 0);
     }
-    if (__any_sync(kAll, rbad || cbad || min(e[0], e[1]) < kSplitSumTiny)) {
+    const bool real = split_real(im);
+    if (__any_sync(kAll, rbad || cbad || split_any_small<KS>(use, real, v) || min(e[0], e[1]) < kSplitSumTiny)) {
+        bool bad[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const bool col_bad = __shfl_sync(kAll, (int)cbad, 8 * t + 4 * j) != 0;
-            if (rbad || col_bad) {
-                // each entry decides for itself, so that it does not depend
-                // on which columns share its tile
-                z2 r = zmk(0.0, 0.0);
-                for (int k = 0; k < 8 * ks; ++k) {
-                    const z2 x = la(g, k), y = lb(2 * t + j, k);
-                    if constexpr (KIND == kConjA) zmac_ca(r, x, y);
-                    else if constexpr (KIND == kPlain) zmac(r, x, y);
-                    else zmac_cb(r, x, y);
-                }
-                v[j] = r;
-                e[j] = 2100;
-            } else if (e[j] < kSplitSumTiny) {
-                // two exact factors down to the last, which rounds into the subnormal range
-                const double s0 = split_scale(2100 - 950), s1 = split_scale(e[j] + 950);
-                v[j].x = v[j].x * s0 * s1;
-                v[j].y = v[j].y * s0 * s1;
-                e[j] = 2100;
-            }
+            const int col_bad = __shfl_sync(kAll, (int)cbad, 8 * t + 4 * j);     // (for all lanes)
+            bad[j] = rbad | (col_bad != 0);
+        }
+        SplitOut o = {{v[0], v[1]}, {e[0], e[1]}};
+        if constexpr (kJoint) o = split_slow<KIND, KS>(ks, la, lb, SplitGridJoint{ea}, use, real, bad[0], bad[1], o);
+        else o = split_slow<KIND, KS>(ks, la, lb, SplitGrid{ea, eb}, use, real, bad[0], bad[1], o);
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            v[j] = o.v[j];
+            e[j] = o.e[j];
         }
     }
 }
 
 // split_tile for operands that are on their grids already: v[j] in units of
-// 2^(Ea + Eb - 54).
+// 2^(Ea + Eb - 54), without a look at small results.
 template <SplitKind KIND, int KS, class LA, class LB>
 __device__ __forceinline__ void split_tile_on(int ks, LA la, LB lb, bool same, z2 (&v)[2]) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
