@@ -58,17 +58,23 @@ __device__ __forceinline__ int tri8_row(int f) {
 // The breakdown test of pivot d of block b, and 1 / d: the approximate reciprocal
 // and one third-order step (y (1 + e + e^2), e = 1 - d y).  Pivots in
 // 2^-999 .. 2^985 are told by their high word, as a comparison in FP64 would
-// take as long as a step of the reciprocal.
+// take as long as a step of the reciprocal.  0 for the others, whose
+// reciprocal need not be a normal number: pivot_scale divides by them.
 __device__ __forceinline__ double pivot_rcp(const LevelArgs &a, int64_t block, double d) {
     if ((unsigned)(__double2hiint(d) - 0x01800000) >= 0x7c000000u) {
         if (!(d > 0.0)) report_fail(a.status, a.level, report_index(a, 2 * block));
-        return 1.0 / d;
+        return 0.0;
     }
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
     double e = fma(-d, y, 1.0);
     e = fma(e, e, e);
     return fma(y, e, y);
+}
+
+// v / d for pivot d with reciprocal s (pivot_rcp).
+__device__ __forceinline__ z2 pivot_scale(z2 v, double d, double s) {
+    return __double2hiint(s) != 0 ? zscale(v, s) : zmk(v.x / d, v.y / d);
 }
 
 // X = L^{-1} of the diagonal blocks o .. o + w - 1 (w <= 8) of A_b = L L^H (packed
@@ -111,8 +117,9 @@ __device__ __forceinline__ void chol_inv8(const LevelArgs &a, int64_t t0, z2 *sL
                 const double s = pivot_rcp(a, t0 + b, d);
                 if (c + 1 >= w) break;
                 z2 t, wv[2];
-                t.x = __shfl_sync(kAll, col.x, 4 * r + (c >> 1)) * s;
-                t.y = __shfl_sync(kAll, col.y, 4 * r + (c >> 1)) * s;
+                t.x = __shfl_sync(kAll, col.x, 4 * r + (c >> 1));
+                t.y = __shfl_sync(kAll, col.y, 4 * r + (c >> 1));
+                t = pivot_scale(t, d, s);
                 const z2 cc = zconj(col);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -157,11 +164,11 @@ __device__ __forceinline__ void chol_inv8(const LevelArgs &a, int64_t t0, z2 *sL
             for (int b = b1; b < nbh; b += q1) {
                 const z2 *Lb = sL + b * SL;
                 z2 *Cb = sC + b * SC;
-                const double s = Lb[at(c, c)].y;
+                const z2 p = Lb[at(c, c)];
                 for (int i = f1; i < w; i += s1) {
                     if (i <= c) continue;
                     const z2 v = Lb[at(i, c)];
-                    Cb[i] = zscale(v, s);
+                    Cb[i] = pivot_scale(v, p.x, p.y);
                     Cb[8 + i] = v;
                 }
             }
