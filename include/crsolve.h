@@ -178,8 +178,8 @@ int crsolve_set_scratch(crsolve_plan p, void *dev_ptr, size_t bytes);
  *   stream: one kernel per level, plus a fix-up kernel for the CTA-boundary
  *   blocks on levels of more than four CTAs per SM.  Systems of N < 8192 and
  *   m <= 32 run their coarse levels in one kernel (and the solve's two sweeps of
- *   them in another), counted and timed under the finest of these levels as
- *   CRSOLVE_K_FACTOR_ODD and CRSOLVE_K_SOLVE_DOWN_ODD.
+ *   them in another) with the same numbers; while kernels are timed
+ *   (crsolve_timing_enable) each level has kernels of its own there too.
  *   Accuracy of the FP64 form: blocks of m <= 6 and m = 9, 10 use FMAs and
  *   substitutions.  The products of the others are formed from 57-bit
  *   fixed-point operands on the tensor cores and rounded once; a result much

@@ -395,11 +395,12 @@ unsigned *boundary_counters(crsolve_plan_s *p, int64_t need, cudaStream_t s, int
 // kTailMaxN blocks only: there the coarse levels are most of the time
 // (N = 64, m = 4, k = 1 solved once: 229 us by levels, 194 so; forward and backward at
 // N = 1024, m = 12, k = 2: 830 and 772), and longer systems
-// keep one launch per level, which callers of the launch counter rely on.
+// keep one launch per level, which callers of the launch counter rely on.  None
+// while kernels are timed: the records are per level and kernel.
 constexpr int64_t kTailMaxN = 8192;
 int tail_level(const crsolve_plan_s *p, int l0) {
     const int nlev = (int)p->lev.size();
-    if (p->N >= kTailMaxN) return nlev;
+    if (p->N >= kTailMaxN || p->timing) return nlev;
     int l = l0;
     while (l < nlev && p->lev[l].no > crs::kTailCtas * (int64_t)crs::tail_blocks(p->m)) ++l;
     return nlev - l >= 2 ? l : nlev;
