@@ -1,12 +1,13 @@
 """Tile autotuner of the batched form and of the single-system plans.
 
 Batched form: for every block-size class MT (4, 8, 16, 32, 64) present in a
-batch, it times the persistent batched kernel on a sample batch of that class
+batch, it times the persistent batched kernel on a sample batch of that class,
+which takes as many threads per CTA as the batch does (see batch_threads),
 and keeps the fastest (odd blocks per chunk in the factor step, odd blocks
 per chunk in the solve steps, right-hand-side columns per chunk).  Plans
 (plan_tiles): per class, width k and precision, a coordinate search over the
 five parameters of the plan kernels' tile table.  Results are cached per GPU
-name in _build/tiles.json next to the library.  The sample inputs come from
+name and library sources in _build/tiles.json next to the library.  The sample inputs come from
 torch's generator (their values do not matter for timing, only their shapes;
 they are diagonally dominant, so every sample factorises).
 """
@@ -31,6 +32,19 @@ def _mt(m: int) -> int:
         if m <= c:
             return c
     raise ValueError("m > 64")
+
+
+def _form(m: int) -> str:
+    """The kernels' form of an FP64 block size (split_form in cr_core64.cuh)."""
+    return "split" if m >= 11 or m in (7, 8) else "fma"
+
+
+def batch_threads(Ns, ms, ks, nsm: int) -> int:
+    """Threads per CTA that crsolve_batch_create takes for a batch: 512 where the
+    largest system has more than its share of two CTAs per SM."""
+    Ns, ms, ks = (np.asarray(v, np.float64) for v in (Ns, ms, ks))
+    cost = Ns * (25.33 * ms ** 3 + 40.0 * ms ** 2 * ks)
+    return 512 if cost.max() * 2 * nsm > cost.sum() else 256
 
 
 def _sample_inputs(Ns, ms, ks, device):
@@ -66,11 +80,12 @@ def _time(b: Batch, A, B, y, x, reps=3) -> float:
     return e0.elapsed_time(e1) / reps
 
 
-def tune_class(mt: int, m: int, k: int, device=None, n_blocks: int = 512, verbose: bool = False):
-    """Best (nb_factor, nb_solve, kc) for class mt on systems of size m, width k."""
+def tune_class(mt: int, m: int, k: int, device=None, n_blocks: int = 512, verbose: bool = False, threads: int = 256):
+    """Best (nb_factor, nb_solve, kc) for class mt on systems of size m, width k, in
+    a batch that runs CTAs of `threads` threads (batch_threads)."""
     device = device or torch.device("cuda", torch.cuda.current_device())
     nslots_guess = torch.cuda.get_device_properties(device).multi_processor_count * 2
-    nsys = 2 * nslots_guess
+    nsys = 2 * nslots_guess if threads == 256 else nslots_guess - 1
     Ns = np.full(nsys, n_blocks, np.int64)
     ms = np.full(nsys, m, np.int32)
     ks = np.full(nsys, k, np.int32)
@@ -116,21 +131,23 @@ def load_cache():
         return {}
 
 
-def tiles_for(ms, ks, device=None, use_cache: bool = True, verbose: bool = False):
-    """{mt: (nb_factor, nb_solve, kc)} for the classes present in a batch."""
+def tiles_for(ms, ks, device=None, use_cache: bool = True, verbose: bool = False, threads: int = 256):
+    """{mt: (nb_factor, nb_solve, kc)} for the classes present in a batch that runs
+    CTAs of `threads` threads.  Cached by what the timings depend on: the GPU, the
+    library's sources, the class, the form of its largest block and the threads."""
     device = device or torch.device("cuda", torch.cuda.current_device())
-    name = torch.cuda.get_device_name(device)
+    name = f"{torch.cuda.get_device_name(device)}|{_build.source_hash()}"
     cache = load_cache() if use_cache else {}
     out, changed = {}, False
     ms = np.asarray(ms)
     ks = np.asarray(ks)
     for mt in sorted({_mt(int(m)) for m in ms}):
-        key = f"{name}|mt={mt}"
+        sel = np.array([_mt(int(m)) == mt for m in ms])
+        m_rep = int(np.max(ms[sel]))
+        key = f"{name}|mt={mt}|{_form(m_rep)}|threads={threads}"
         if key not in cache:
-            sel = np.array([_mt(int(m)) == mt for m in ms])
-            m_rep = int(np.max(ms[sel]))
             k_rep = int(np.median(ks[sel]))
-            best, table = tune_class(mt, m_rep, k_rep, device, verbose=verbose)
+            best, table = tune_class(mt, m_rep, k_rep, device, verbose=verbose, threads=threads)
             cache[key] = {"tile": best, "m": m_rep, "k": k_rep, "timings_ms": table}
             changed = True
         out[mt] = tuple(cache[key]["tile"])
@@ -147,7 +164,7 @@ def tiles_for(ms, ks, device=None, use_cache: bool = True, verbose: bool = False
 # precision (crsolve_tile_set / crsolve_tile_set_mixed).  plan_tiles() picks a
 # shape for (class, k, precision) by timing factor + solve of a sample system
 # over the candidates (each parameter around the current shape, a coordinate
-# search), caches it per GPU name under that key, and with apply=True writes
+# search), caches it per GPU name and library sources under that key, and with apply=True writes
 # it into the table for later launches of every plan of that class.
 
 PLAN_NB = (1, 2, 4, 8, 16, 32)
@@ -230,13 +247,14 @@ def tune_plan_class(m: int, k: int, precision: int = 0, n_blocks: int = 0, devic
 def plan_tiles(m: int, k: int, precision: int = 0, device=None, use_cache: bool = True, apply: bool = True,
                verbose: bool = False):
     """The tuned tile shape of class mt(m) for width k and precision, from the
-    cache (key: GPU name, class, k rounded up to a power of two, precision)
+    cache (key: GPU name, library sources, class, form, k rounded up to a power of
+    two, precision)
     or tuned now; with apply=True it is written into the process-wide table."""
     from . import api
     device = device or torch.device("cuda", torch.cuda.current_device())
-    name = torch.cuda.get_device_name(device)
+    name = f"{torch.cuda.get_device_name(device)}|{_build.source_hash()}"
     kb = 1 << max(0, (int(k) - 1).bit_length())
-    key = f"{name}|plan|mt={_mt(m)}|k={kb}|prec={'mixed' if precision else 'fp64'}"
+    key = f"{name}|plan|mt={_mt(m)}|{_form(m)}|k={kb}|prec={'mixed' if precision else 'fp64'}"
     cache = load_cache() if use_cache else {}
     if key not in cache:
         best, table = tune_plan_class(m, kb, precision, device=device, verbose=verbose)

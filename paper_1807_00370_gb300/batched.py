@@ -39,8 +39,9 @@ class Batch:
         if isinstance(tiles, str):
             if tiles != "auto":
                 raise ValueError("tiles must be None, 'auto' or {mt: (nb_factor, nb_solve, kc)}")
-            from .autotune import tiles_for
-            tiles = tiles_for(self.ms, self.ks, self.device)
+            from .autotune import batch_threads, tiles_for
+            nsm = torch.cuda.get_device_properties(self.device).multi_processor_count
+            tiles = tiles_for(self.ms, self.ks, self.device, threads=batch_threads(self.Ns, self.ms, self.ks, nsm))
         self.tiles = dict(tiles or {})
         self.nsys = len(self.Ns)
         self._h = ctypes.c_void_p()

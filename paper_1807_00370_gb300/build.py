@@ -7,6 +7,7 @@ Every translation unit under csrc/ is compiled in parallel with
 from __future__ import annotations
 
 import glob
+import hashlib
 import os
 import subprocess
 import sys
@@ -37,6 +38,15 @@ def _sources():
 def _deps():
     return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
         glob.glob(os.path.join(INCLUDE, "*.h")) + [os.path.abspath(__file__)]
+
+
+def source_hash() -> str:
+    """Short hash of everything the library is built from (names what was timed)."""
+    h = hashlib.sha256()
+    for d in sorted(_deps()):
+        with open(d, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:12]
 
 
 def is_stale(debug: bool = False) -> bool:
