@@ -378,6 +378,11 @@ constexpr int kWsXStage = 8 * kRtNC * 16;                  // 4096 bytes: the ra
 constexpr int kWsStage = kWsAStage + kWsBStage + kWsXStage;
 constexpr int kWsStages = 4;
 constexpr int kWsSlicers = 192, kWsEpi = 256;
+// Exponent sets kept: the slicers write that of pass P once chunk kWsChunks -
+// kWsStages of pass P - 1 is done, so once the epilogue has read the accumulators
+// of pass P - 2, that is, ended pass P - 3.  It reads the exponents after the
+// accumulators, so the set of pass P - 2 may still be in use then: a third one.
+constexpr int kWsSlots = 3;
 static_assert(kWsChunks * kWsAStage == 12 * kRtAStage, "image bytes per block row");
 
 // Byte offset of element (r, k) of a K-major, unswizzled tile of 16-bit
@@ -456,8 +461,8 @@ __global__ void __launch_bounds__(kRtThreads, 1) k_residual_ws(ResidTcArgs a) {
     uint64_t *accfull = xr + kWsStages, *accempty = accfull + 1;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(accempty + 1);
     volatile int *sAbort = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    int *sEr = reinterpret_cast<int *>(tmem_slot + 4);          // [2][64]
-    int *sEc = sEr + 128;                                        // [2][32]
+    int *sEr = reinterpret_cast<int *>(tmem_slot + 4);          // [kWsSlots][64]
+    int *sEc = sEr + kWsSlots * 64;                              // [kWsSlots][32]
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int m = a.m, k = a.k;
@@ -578,10 +583,10 @@ __global__ void __launch_bounds__(kRtThreads, 1) k_residual_ws(ResidTcArgs a) {
                 break;
             }
             const int64_t P = G / kWsChunks, j = row_of(P);
-            const int c = (int)(G % kWsChunks), col0 = (int)(P % npass) * kRtNC, slot = (int)(P & 1);
+            const int c = (int)(G % kWsChunks), col0 = (int)(P % npass) * kRtNC, slot = (int)(P % kWsSlots);
             if (c == 0) {
                 // the pass's exponents (its slot was last read by the epilogue of
-                // pass P - 2, which ended before any MMA of pass P - 1)
+                // pass P - 3: see kWsSlots)
                 if (sid < 64) sEr[slot * 64 + sid] = sid < m ? a.erow[j * m + sid] : kExpZero;
                 if (sid >= 64 && sid < 64 + kRtNC) {
                     const int cc = sid - 64, col = col0 + cc;
@@ -640,7 +645,7 @@ __global__ void __launch_bounds__(kRtThreads, 1) k_residual_ws(ResidTcArgs a) {
         };
         for (int64_t P = 0; P < passes; ++P) {
             const int64_t j = row_of(P);
-            const int col0 = (int)(P % npass) * kRtNC, slot = (int)(P & 1);
+            const int col0 = (int)(P % npass) * kRtNC, slot = (int)(P % kWsSlots);
             if (!wait_or_abort(smem_u32(accfull), (uint32_t)P & 1u, sAbort)) {
                 *sAbort = 1;
                 break;
@@ -915,7 +920,8 @@ __global__ void __launch_bounds__(kRtThreads, 1) k_residual_tc(ResidTcArgs a) {
 }  // namespace
 
 size_t residual_tc_smem_bytes() { return 2 * (size_t)kRtStage + 1024 + 1024; }
-static size_t residual_ws_smem_bytes() { return kWsStages * (size_t)kWsStage + 1024 + 1024; }
+// stages, alignment, then barriers (under 256 bytes) and the exponent sets
+static size_t residual_ws_smem_bytes() { return kWsStages * (size_t)kWsStage + 1024 + 256 + kWsSlots * (64 + 32) * 4; }
 
 size_t residual_image_bytes(int64_t N) { return (size_t)N * kWsChunks * (size_t)kWsAStage; }
 
