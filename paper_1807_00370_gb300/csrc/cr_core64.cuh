@@ -55,21 +55,16 @@ __device__ __forceinline__ int tri8_row(int f) {
     return f >= 28 ? 7 : __popc(kStarts & ((2u << f) - 1u));
 }
 
-// The breakdown test of pivot d of block b, and 1 / d: the approximate reciprocal
-// and one third-order step (y (1 + e + e^2), e = 1 - d y).  Pivots in
-// 2^-999 .. 2^985 are told by their high word, as a comparison in FP64 would
+// The breakdown test of pivot d of block b, and 1 / d (fast_rcp).  Pivots in
+// fast_rcp's range are told by their high word, as a comparison in FP64 would
 // take as long as a step of the reciprocal.  0 for the others, whose
 // reciprocal need not be a normal number: pivot_scale divides by them.
 __device__ __forceinline__ double pivot_rcp(const LevelArgs &a, int64_t block, double d) {
-    if ((unsigned)(__double2hiint(d) - 0x01800000) >= 0x7c000000u) {
+    if (!fast_rcp_takes(d)) {
         if (!(d > 0.0)) report_fail(a.status, a.level, report_index(a, 2 * block));
         return 0.0;
     }
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-    double e = fma(-d, y, 1.0);
-    e = fma(e, e, e);
-    return fma(y, e, y);
+    return fast_rcp(d);
 }
 
 // v / d for pivot d with reciprocal s (pivot_rcp).

@@ -49,3 +49,13 @@ extern "C" int split_tile_device(int kind, int ks, const void *a, const void *b,
     if (kind == 1) return tile_ks<kPlain, true>(ks, pa, pb, po);
     return tile_ks<kConjB, true>(ks, pa, pb, po);
 }
+
+// r[i] = fast_rcp(d[i]) where it takes d[i], else 0; device pointers.
+__global__ void k_rcp(const double *d, double *r, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) r[i] = fast_rcp_takes(d[i]) ? fast_rcp(d[i]) : 0.0;
+}
+extern "C" int fast_rcp_device(const void *d, void *r, int n) {
+    k_rcp<<<(n + 255) / 256, 256>>>(static_cast<const double *>(d), static_cast<double *>(r), n);
+    return (int)cudaDeviceSynchronize();
+}
