@@ -46,6 +46,22 @@ struct TailArgs {
     LevelArgs lev[kTailLevels];
 };
 int tail_blocks(int m);
+
+// Cost of one refinement step of the mixed form (an FP32 correction sweep and an
+// FP64-accurate product) relative to the FP64 factor + solve.
+// split (tensor-core residuals, m > 32): 8.5 / m, fitted to times at N = 2048 and at
+// full size, k = 1 .. 32: m = 33 0.21 .. 0.25, m = 40 0.20 .. 0.23, m = 48 0.16 .. 0.18,
+// m = 64 0.13 .. 0.14 (6.8 of 48.5 ms at N = 16384, k = 32).
+// FP64-pipe residuals: by FP64-pipe flops per block row, 24 m^2 k of the product and
+// an eighth of the sweep's 40 m^2 k against 25.33 m^3 + 40 m^2 k of the FP64 path by
+// FMAs.  Against the tensor-core FP64 path a step takes more (0.2 .. 1.1 of it at
+// m = 24, 0.3 .. 2.3 at m = 8); the count is kept, as it decides which calls
+// end refined and which in FP64.
+inline double mixed_step_cost(int m, int k, bool split) {
+    if (split) return 8.5 / m;
+    const double mm = (double)m * m;
+    return (24.0 + 5.0) * mm * k / (25.33 * mm * m + 40.0 * mm * k);
+}
 cudaError_t prepare_tail(int m, int smem_optin);
 cudaError_t launch_factor_tail(const TailArgs &ta, cudaStream_t s);
 cudaError_t launch_solve_tail(const TailArgs &ta, cudaStream_t s);

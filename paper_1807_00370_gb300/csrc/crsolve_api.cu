@@ -901,16 +901,6 @@ int mixed_correction(crsolve_plan_s *p, int k, const z2 *r, cudaStream_t s) {
 // corrections down to 1e-16, error 2.8e-9 against the oracle.
 constexpr double kMixedTol = 1e-11, kMixedExtrapFrom = 1e-8, kMixedVerifyAbove = 1e-4;
 
-// Cost of one step (an FP32 correction sweep and an FP64-accurate product)
-// relative to the FP64 factor + solve, in FP64-pipe flops per block row:
-// the FP32 sweep 40 m^2 k flop at about 1/8 of its FP64 time (measured), the
-// product 24 m^2 k flop on the FP64 pipe, or about 1/16 of that with the
-// tensor-core splitting; the FP64 path 25.33 m^3 + 40 m^2 k.
-double mixed_step_cost(int m, int k, bool split) {
-    const double mm = (double)m * m, step = (split ? 1.5 : 24.0) * mm * k + 5.0 * mm * k;
-    return step / (25.33 * mm * m + 40.0 * mm * k);
-}
-
 // r = y - A x (y may be NULL: r = -A x), FP64-accurate.
 int mixed_residual(crsolve_plan_s *p, int k, const z2 *x, const z2 *y, z2 *r, cudaStream_t s) {
     const WsMap ws = p->map();
@@ -1042,7 +1032,7 @@ int mixed_solve(crsolve_plan_s *p, int k, const z2 *y, z2 *x, cudaStream_t s) {
             if (rho < 1.0) {
                 // steps still needed for rho^n * delta <= kMixedTol, against the FP64 path
                 const double need = std::ceil(std::log(kMixedTol / (rho * delta)) / std::log(rho));
-                if (need * mixed_step_cost(p->m, k, mixed_uses_split(p)) > 1.0) break;
+                if (need * crs::mixed_step_cost(p->m, k, mixed_uses_split(p)) > 1.0) break;
             }
         }
         prev = delta;

@@ -1,5 +1,6 @@
 // Entry points to the pieces of cr_split.cuh for the tests that compare them
 // with exact integer and rational arithmetic.
+#include "cr_launch.h"
 #include "cr_split.cuh"
 
 using namespace crs;
@@ -59,3 +60,5 @@ extern "C" int fast_rcp_device(const void *d, void *r, int n) {
     k_rcp<<<(n + 255) / 256, 256>>>(static_cast<const double *>(d), static_cast<double *>(r), n);
     return (int)cudaDeviceSynchronize();
 }
+
+extern "C" double mixed_step_cost_host(int m, int k, int split) { return mixed_step_cost(m, k, split != 0); }

@@ -14,4 +14,5 @@ def load(tmp_dir):
                     os.path.join(HERE, "device", "split_check.cu")], check=True)
     lib = ctypes.CDLL(so)
     lib.split_value_host.restype = ctypes.c_double
+    lib.mixed_step_cost_host.restype = ctypes.c_double
     return lib
