@@ -362,22 +362,26 @@ struct SplitSeen {
     }
 };
 
-// A lane's entries (g, 2t + j) with fma[j] by FMAs over n terms (n a multiple of 8).
+// A lane's entries (g, 2t + j) with fma[j] by FMAs over the K-steps in steps (bits).
 // The warp goes through the terms together, without a branch on fma.
 template <SplitKind KIND, class LA, class LB>
-__device__ __forceinline__ void split_entries(int n, LA la, LB lb, const bool (&fma)[2], z2 (&v)[2], int (&ex)[2]) {
+__device__ __forceinline__ void split_entries(int ks, unsigned steps, LA la, LB lb, const bool (&fma)[2], z2 (&v)[2], int (&ex)[2]) {
     const int lane = threadIdx.x & 31, g = lane >> 2, c = 2 * (lane & 3);
     if (!__any_sync(0xffffffffu, fma[0] | fma[1])) return;
     z2 r[2] = {zmk(0.0, 0.0), zmk(0.0, 0.0)};
+#pragma unroll 1
+    for (int s = 0; s < ks; ++s) {
+        if (!(steps >> s & 1u)) continue;
 #pragma unroll 4
-    for (int k = 0; k < n; ++k) {
-        const z2 x = la(g, k);
+        for (int k = 8 * s; k < 8 * s + 8; ++k) {
+            const z2 x = la(g, k);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const z2 y = lb(c + j, k);
-            if constexpr (KIND == kConjA) zmac_ca(r[j], x, y);
-            else if constexpr (KIND == kPlain) zmac(r[j], x, y);
-            else zmac_cb(r[j], x, y);
+            for (int j = 0; j < 2; ++j) {
+                const z2 y = lb(c + j, k);
+                if constexpr (KIND == kConjA) zmac_ca(r[j], x, y);
+                else if constexpr (KIND == kPlain) zmac(r[j], x, y);
+                else zmac_cb(r[j], x, y);
+            }
         }
     }
 #pragma unroll
@@ -407,13 +411,18 @@ struct SplitGridJoint {     // rows of exponent sum ea on the terms' own
 };
 
 // Which of a lane's entries with small parts (bits of split_small) to form by FMAs.
-// For all lanes of a warp.
+// For all lanes of a warp.  Returns the K-steps (bits, the same in all lanes) that
+// have a nonzero product for such an entry: blocks of triangular and banded operands
+// have them in few.
 template <class LA, class LB, class GRID>
-__device__ __forceinline__ void split_guard(int ks, LA la, LB lb, GRID grid, const unsigned (&small)[2], bool (&need)[2]) {
+__device__ __forceinline__ unsigned split_guard(int ks, LA la, LB lb, GRID grid, const unsigned (&small)[2], bool (&need)[2]) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     SplitSeen seen;
+    unsigned steps = 0;
+    const unsigned mine = (small[0] ? 3u : 0u) | (small[1] ? 12u : 0u);     // (both parts of an entry are formed)
 #pragma unroll 1
     for (int s = 0; s < ks; ++s) {
+        SplitSeen now;
         z2 a[2], b[2];
         int ea[2], eb[2];
 #pragma unroll
@@ -423,10 +432,14 @@ __device__ __forceinline__ void split_guard(int ks, LA la, LB lb, GRID grid, con
         }
         grid(s, b[0], b[1], ea, eb);
 #pragma unroll
-        for (int u = 0; u < 2; ++u) seen.term(a[u], ea[u], b[u], eb[u]);
+        for (int u = 0; u < 2; ++u) now.term(a[u], ea[u], b[u], eb[u]);
+        seen.nz |= now.nz;
+        seen.big |= now.big;
+        if (__any_sync(0xffffffffu, (now.nz & mine) != 0u)) steps |= 1u << s;
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j) need[j] = (small[j] & ((seen.nz & ~seen.big) >> (2 * j))) != 0u;
+    return steps;
 }
 
 // The imaginary part of an operand as bits, 0: none.
@@ -486,7 +499,9 @@ __device__ __noinline__ SplitOut split_slow(int ks, LA la, LB lb, GRID grid, Spl
     const bool bad[2] = {bad0, bad1};
     bool need[2] = {false, false};
     unsigned small[2];
-    if (split_smalls<KS>(use, real, o.v, small)) split_guard(ks, la, lb, grid, small, need);
+    unsigned steps = 0;
+    if (split_smalls<KS>(use, real, o.v, small)) steps = split_guard(ks, la, lb, grid, small, need);
+    if (__any_sync(0xffffffffu, bad0 | bad1)) steps = 0xffffffffu;      // (zeros times infinity or NaN count)
     // each entry decides for itself, so that it does not depend on which
     // columns share its tile
 #pragma unroll
@@ -500,7 +515,7 @@ __device__ __noinline__ SplitOut split_slow(int ks, LA la, LB lb, GRID grid, Spl
             o.e[j] = 2100;
         }
     }
-    split_entries<KIND>(8 * ks, la, lb, need, o.v, o.e);
+    split_entries<KIND>(ks, steps, la, lb, need, o.v, o.e);
     __syncwarp();
     return o;
 }
