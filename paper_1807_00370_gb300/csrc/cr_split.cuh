@@ -363,15 +363,26 @@ struct SplitSeen {
 };
 
 // A lane's entries (g, 2t + j) with fma[j] by FMAs over the K-steps in steps (bits).
-// The warp goes through the terms together, without a branch on fma.
+// The warp goes through the terms together, without a branch on fma.  real: all
+// operands are real, one FMA per term instead of four.
 template <SplitKind KIND, class LA, class LB>
-__device__ __forceinline__ void split_entries(int ks, unsigned steps, LA la, LB lb, const bool (&fma)[2], z2 (&v)[2], int (&ex)[2]) {
+__device__ __forceinline__ void split_entries(int ks, unsigned steps, LA la, LB lb, bool real, const bool (&fma)[2], z2 (&v)[2],
+                                              int (&ex)[2]) {
     const int lane = threadIdx.x & 31, g = lane >> 2, c = 2 * (lane & 3);
     if (!__any_sync(0xffffffffu, fma[0] | fma[1])) return;
     z2 r[2] = {zmk(0.0, 0.0), zmk(0.0, 0.0)};
 #pragma unroll 1
     for (int s = 0; s < ks; ++s) {
         if (!(steps >> s & 1u)) continue;
+        if (real) {
+#pragma unroll
+            for (int k = 8 * s; k < 8 * s + 8; ++k) {
+                const double x = la(g, k).x;
+#pragma unroll
+                for (int j = 0; j < 2; ++j) r[j].x = ::fma(x, lb(c + j, k).x, r[j].x);
+            }
+            continue;
+        }
 #pragma unroll 4
         for (int k = 8 * s; k < 8 * s + 8; ++k) {
             const z2 x = la(g, k);
@@ -501,7 +512,8 @@ __device__ __noinline__ SplitOut split_slow(int ks, LA la, LB lb, GRID grid, Spl
     unsigned small[2];
     unsigned steps = 0;
     if (split_smalls<KS>(use, real, o.v, small)) steps = split_guard(ks, la, lb, grid, small, need);
-    if (__any_sync(0xffffffffu, bad0 | bad1)) steps = 0xffffffffu;      // (zeros times infinity or NaN count)
+    const bool any_bad = __any_sync(0xffffffffu, bad0 | bad1);
+    if (any_bad) steps = 0xffffffffu;       // (zeros times infinity or NaN count)
     // each entry decides for itself, so that it does not depend on which
     // columns share its tile
 #pragma unroll
@@ -515,7 +527,7 @@ __device__ __noinline__ SplitOut split_slow(int ks, LA la, LB lb, GRID grid, Spl
             o.e[j] = 2100;
         }
     }
-    split_entries<KIND>(ks, steps, la, lb, need, o.v, o.e);
+    split_entries<KIND>(ks, steps, la, lb, real && !any_bad, need, o.v, o.e);
     __syncwarp();
     return o;
 }
