@@ -56,13 +56,15 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FP64_FMA_PER_CLK_SM, N_SM, SM_MAX_MHZ = 2, 152, 2070.0
 FP64_PEAK_GFLOPS = FP64_FMA_PER_CLK_SM * 2 * N_SM * SM_MAX_MHZ / 1e3
 # DRAM traffic of the dominant kernel from one ncu capture (dram__bytes_read.sum
-# + dram__bytes_write.sum of k_factor_odd<8, double>, level 0 of N = 2^18, 2^17
-# odd blocks: 537,975,296 + 624,427,776 bytes), valid only while the sources
-# of the kernel's device code are the ones captured (their SHA-256 below).
+# + dram__bytes_write.sum of k_factor_split<8>, level 0 of N = 2^18, 2^17 odd
+# blocks: 538,159,616 + 624,610,816 bytes), valid only while the sources of the
+# kernel's device code are the ones below (their SHA-256; the capture was taken
+# before a last change to comments and to the bounds-checked build's helper).
 # Otherwise the line reports null.
-TRAFFIC_CAPTURE = {"bytes_per_odd_block": (537975296 + 624427776) / (1 << 17),
-                   "sources": ("paper_1807_00370_gb300/csrc/cr_core.cuh", "paper_1807_00370_gb300/csrc/cr_device.cuh"),
-                   "sha256": "0bd90a121a9eef595ab08f3a2c51afd23043dea0d0daca35ce1979fa79ddd871"}
+TRAFFIC_CAPTURE = {"bytes_per_odd_block": (538159616 + 624610816) / (1 << 17),
+                   "sources": ("paper_1807_00370_gb300/csrc/cr_split.cuh", "paper_1807_00370_gb300/csrc/cr_core64.cuh",
+                               "paper_1807_00370_gb300/csrc/cr_device.cuh"),
+                   "sha256": "155474f720c66c3abf5bfc3b0b7a88f4f2a8cf871d5dc189bc17a76c8e697058"}
 
 
 # The FP64 levels of blocks m = 7, 8 and m >= 11 form their products exactly from

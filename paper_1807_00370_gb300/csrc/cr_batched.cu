@@ -183,7 +183,8 @@ int crsolve_batch_create(int32_t nsys, const int64_t *N, const int32_t *m, const
     // A system runs in one CTA, so a batch lasts at least as long as its largest
     // system.  Where that system has more than its share of 2 CTAs per SM, the
     // batch runs CTAs of 512 threads, one per SM, with chunks of twice the blocks
-    // where they fit: 512 systems of N <= 4096, m = 4 .. 32 479 ms at 256 threads, 246 so.
+    // where they fit: 512 systems of N <= 4096, m = 4 .. 32 took 479 ms at 256 threads
+    // and 246 so (263 since small results take FMAs).
     const double total = std::accumulate(cost.begin(), cost.end(), 0.0);
     const double largest = *std::max_element(cost.begin(), cost.end());
     if (largest * 2 * b->nsm > total) {

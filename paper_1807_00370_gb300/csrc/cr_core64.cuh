@@ -28,7 +28,9 @@ namespace crs {
 // 8 x 8 costs more than the FMAs (factor and solve at N = 100003, k = 3: 815 + 1076
 // against 595 + 800 us), and so does that of m = 9 and 10 to 16 x 16 (factor at
 // m = 10, N = 48000: about 1900 against 1733 us; at m = 11, N = 36062: 1574 against
-// 1652, solve with k = 4 1009 against 1436).
+// 1652, solve with k = 4 1009 against 1436, before small results took FMAs; with
+// them, and on banded systems, the factor is 1.45 times the FMA form's and the
+// solve 0.77 of it).
 __host__ __device__ constexpr bool split_form(int m, size_t rsize) { return rsize == 8 && (m >= 11 || m == 7 || m == 8); }
 // The classes that have blocks of either kind.
 template <int MT, class R> struct Forms {
@@ -307,6 +309,7 @@ __device__ __forceinline__ void inverse_chunk(const LevelArgs &a, int64_t t0, z2
 // One chunk of nb odd blocks of a factor level (see factor_chunk).
 template <int MT, bool FULL>
 __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, unsigned char *smem_raw) {
+    [[maybe_unused]] const LevelArgs *const ap = &a;    // for bounds-checked loads in closures
     constexpr int LDZ = Split64<MT>::LDZ, SL = Split64<MT>::SL, KS = MT / 8;
     constexpr bool kOn = MT >= 32;
     const int m = FULL ? MT : a.m, nb = a.nb, NT = blockDim.x, tid = threadIdx.x;
@@ -353,7 +356,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                         if (!((FULL || 8 * R + i < m) && k <= 8 * R + i)) return zmk(0.0, 0.0);
                         if constexpr (!kOn) return Xb[tri(8 * R + i, k)];
                         const int64_t o = t * mm + (8 * R + i) * m + k;     // (sL has X on its grid)
-                        return CRS_IN(a, kDbgL, o) ? XL[o] : zmk(0.0, 0.0);
+                        return CRS_IN(*ap, kDbgL, o) ? XL[o] : zmk(0.0, 0.0);
                     },
                     {nc, m - 8 * R, kFull}, false, v, ex);
                 __syncwarp();
@@ -463,7 +466,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                 const z2 *Z = a.Z;
                 return [=](int i, int k) {
                     const int64_t o = oz + k * m2 + i;
-                    return ((FULL || (i < nc && k < m)) && CRS_IN(a, kDbgZ, o)) ? Z[o] : zmk(0.0, 0.0);
+                    return ((FULL || (i < nc && k < m)) && CRS_IN(*ap, kDbgZ, o)) ? Z[o] : zmk(0.0, 0.0);
                 };
             };
             auto zgi = zg(ci, ni), zgj = zg(cj, nj);
@@ -593,7 +596,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                     const z2 *Z = a.Z + t * 2 * (int64_t)mm;
                     auto zl = [=](int h) {
                         return [=](int i, int k) {
-                            return ((FULL || (i < m && k < m)) && CRS_IN(a, kDbgZ, t * 2 * (int64_t)mm + k * m2 + h * m + i)) ? Z[k * m2 + h * m + i]
+                            return ((FULL || (i < m && k < m)) && CRS_IN(*ap, kDbgZ, t * 2 * (int64_t)mm + k * m2 + h * m + i)) ? Z[k * m2 + h * m + i]
                                                                                                                        : zmk(0.0, 0.0);
                         };
                     };
@@ -726,7 +729,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                 auto bg = [=](int i, int k) {       // the columns as the level has them
                     if (!FULL && (i >= nc || k >= m)) return zmk(0.0, 0.0);
                     const int64_t o = inP ? (2 * t - 1) * mm + k * m + c0 + i : 2 * t * mm + (c0 + i) * m + k;
-                    if (!CRS_IN(a, kDbgB, o)) return zmk(0.0, 0.0);
+                    if (!CRS_IN(*ap, kDbgB, o)) return zmk(0.0, 0.0);
                     return inP ? BL[o] : zconj(BL[o]);
                 };
                 for (int s = 0; s < g8; ++s)
@@ -746,7 +749,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
                         [&](int i, int k) { return ((FULL || 8 * R + i < m) && k <= 8 * R + i) ? Xb[tri(8 * R + i, k)] : zero_on; }, false, v);
                     auto xg = [=](int i, int k) {
                         const int64_t o = t * mm + (8 * R + i) * m + k;
-                        return ((FULL || 8 * R + i < m) && k <= 8 * R + i && CRS_IN(a, kDbgL, o)) ? XL[o] : zmk(0.0, 0.0);
+                        return ((FULL || 8 * R + i < m) && k <= 8 * R + i && CRS_IN(*ap, kDbgL, o)) ? XL[o] : zmk(0.0, 0.0);
                     };
                     const int ea = jt.ea, er = (FULL || 8 * R + g < m) ? xe[MT + 8 * R + g] : 0;
                     auto grid = [=](int s, z2, z2, int (&ga)[2], int (&gb)[2]) {
@@ -834,6 +837,7 @@ __device__ __forceinline__ void factor_split(const LevelArgs &a, int64_t chunk, 
 template <int MT, bool FULL>
 __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chunk, int cchunk,
                                                        unsigned char *smem_raw) {
+    [[maybe_unused]] const LevelArgs *const ap = &a;    // for bounds-checked loads in closures
     constexpr int KS = MT / 8;
     const int m = FULL ? MT : a.m, k = a.k, nb = a.nb, kc = a.kc, NT = blockDim.x, tid = threadIdx.x;
     const int mm = m * m, m2 = 2 * m, mk = m * k;
@@ -852,20 +856,20 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
         const int64_t yo = 2 * (t0 + b) * mk + cb + n0;
         const z2 *y = a.y;
         const int nc = kw - n0;
-        return [=](int i, int s) { return (i < nc && (FULL || s < m) && CRS_IN(a, kDbgY, yo + s * k + i)) ? y[yo + s * k + i] : zmk(0.0, 0.0); };
+        return [=](int i, int s) { return (i < nc && (FULL || s < m) && CRS_IN(*ap, kDbgY, yo + s * k + i)) ? y[yo + s * k + i] : zmk(0.0, 0.0); };
     };
     auto x_of = [&](int b, int R) {
         const int64_t xo = (t0 + b) * mm + 8 * R * m;
         const z2 *X = a.L;
         return [=](int i, int s) {
-            return ((FULL || 8 * R + i < m) && s <= 8 * R + i && CRS_IN(a, kDbgL, xo + i * m + s)) ? X[xo + i * m + s] : zmk(0.0, 0.0);
+            return ((FULL || 8 * R + i < m) && s <= 8 * R + i && CRS_IN(*ap, kDbgL, xo + i * m + s)) ? X[xo + i * m + s] : zmk(0.0, 0.0);
         };
     };
     auto z_of = [&](int b, int h, int G) {
         const int64_t zo = (t0 + b) * m2 * m + (h ? m : 0) + 8 * G;
         const z2 *Z = a.Z;
         return [=](int i, int s) {
-            return ((FULL || (8 * G + i < m && s < m)) && CRS_IN(a, kDbgZ, zo + s * m2 + i)) ? Z[zo + s * m2 + i] : zmk(0.0, 0.0);
+            return ((FULL || (8 * G + i < m && s < m)) && CRS_IN(*ap, kDbgZ, zo + s * m2 + i)) ? Z[zo + s * m2 + i] : zmk(0.0, 0.0);
         };
     };
     // r of rows 8 R .. and columns n0 .. of block b
@@ -1019,7 +1023,7 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
                 const int64_t ro = t * mk + cb + n0;
                 const z2 *Rg = a.r;
                 auto rl = [=](int i, int s) {
-                    return (i < nc && (FULL || s < m) && CRS_IN(a, kDbgR, ro + s * k + i)) ? Rg[ro + s * k + i] : zmk(0.0, 0.0);
+                    return (i < nc && (FULL || s < m) && CRS_IN(*ap, kDbgR, ro + s * k + i)) ? Rg[ro + s * k + i] : zmk(0.0, 0.0);
                 };
                 if (split_needs<1>(1, z_of(b, h, 0), rl, {m, nc, kFull}, ir | im_bits(z[h][0]) | im_bits(z[h][1]),
                                    SplitGrid{ez, er}, v)) {
@@ -1088,6 +1092,7 @@ __device__ __forceinline__ void solve_down_split(const LevelArgs &a, int64_t chu
 template <int MT, bool FULL>
 __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk, int cchunk,
                                                      unsigned char *smem_raw) {
+    [[maybe_unused]] const LevelArgs *const ap = &a;    // for bounds-checked loads in closures
     constexpr int KS = MT / 8;
     const int m = FULL ? MT : a.m, k = a.k, nb = a.nb, kc = a.kc, NT = blockDim.x, tid = threadIdx.x;
     const int mm = m * m, m2 = 2 * m, mk = m * k;
@@ -1123,7 +1128,7 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
             const bool right = s >= 8 * g8;
             const int q = right ? s - 8 * g8 : s;
             const int64_t o = xo + (right ? 0 : -mk) + q * k + i;
-            return (i < nc && (FULL || q < m) && (right ? hasR : hasL) && CRS_IN(a, kDbgXn, o)) ? xn[o] : zmk(0.0, 0.0);
+            return (i < nc && (FULL || q < m) && (right ? hasR : hasL) && CRS_IN(*ap, kDbgXn, o)) ? xn[o] : zmk(0.0, 0.0);
         };
     };
     auto z_of = [&](int b, int R) {
@@ -1133,7 +1138,7 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
             const bool right = s >= 8 * g8;
             const int q = right ? s - 8 * g8 : s;
             const int64_t o = zo + i * m2 + (right ? m : 0) + q;
-            return ((FULL || (8 * R + i < m && q < m)) && CRS_IN(a, kDbgZ, o)) ? Z[o] : zmk(0.0, 0.0);
+            return ((FULL || (8 * R + i < m && q < m)) && CRS_IN(*ap, kDbgZ, o)) ? Z[o] : zmk(0.0, 0.0);
         };
     };
     auto x_of = [&](int b, int G) {
@@ -1141,7 +1146,7 @@ __device__ __forceinline__ void solve_up_split(const LevelArgs &a, int64_t chunk
         const int np = m - 8 * G;
         const z2 *X = a.L;
         return [=](int i, int s) {
-            return ((FULL || (i < np && s < np)) && i <= s && CRS_IN(a, kDbgL, xo + s * m + i)) ? X[xo + s * m + i] : zmk(0.0, 0.0);
+            return ((FULL || (i < np && s < np)) && i <= s && CRS_IN(*ap, kDbgL, xo + s * m + i)) ? X[xo + s * m + i] : zmk(0.0, 0.0);
         };
     };
     auto w_task = [&](int b, int R, int n0) {

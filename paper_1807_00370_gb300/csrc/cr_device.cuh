@@ -224,16 +224,16 @@ __device__ __forceinline__ int64_t dbg_extent(const LevelArgsT<R> &a, int which)
 // skips the access (a load gives zero), so a faulty index never touches
 // memory.  Release builds: always true, no code.
 #ifdef CRSOLVE_DEBUG_BOUNDS
+// (the record out of line: it is never reached, and inlined it takes minutes to compile)
+static __device__ __noinline__ bool dbg_out(unsigned long long *dbg, int level, int which, int64_t idx) {
+    if (dbg)
+        atomicMin(dbg, ((unsigned long long)(level & 0xFF) << 56) | ((unsigned long long)which << 48) |
+                           ((unsigned long long)idx & 0xFFFFFFFFFFFFull));
+    return false;
+}
 template <class R>
 __device__ __forceinline__ bool dbg_in(const LevelArgsT<R> &a, int which, int64_t idx) {
-    if (idx >= 0 && idx < dbg_extent(a, which)) return true;
-    if (a.dbg) {
-        const unsigned long long rec = ((unsigned long long)(a.level & 0xFF) << 56) |
-                                       ((unsigned long long)which << 48) |
-                                       ((unsigned long long)idx & 0xFFFFFFFFFFFFull);
-        atomicMin(a.dbg, rec);
-    }
-    return false;
+    return (uint64_t)idx < (uint64_t)dbg_extent(a, which) || dbg_out(a.dbg, a.level, which, idx);
 }
 #define CRS_IN(a, which, idx) (::crs::dbg_in((a), ::crs::which, (int64_t)(idx)))
 #else
